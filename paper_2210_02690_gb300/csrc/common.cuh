@@ -179,6 +179,24 @@ __host__ __device__ __forceinline__ int node_multiplicity(const Geom& g, int ix,
   return m;
 }
 
+// Factor of a removed cell's patch (obstacle, 2D): the projector onto the patch's unknowns without
+// an equation (velocity at Q2 nodes of removed cells only, the cell's pressure), whose rows are
+// the identity; the patch smooths only those.  1 at local entry mu when it is such an unknown.
+__device__ __forceinline__ bool patch_entry_dead(const Geom& g, int cx, int cy, int mu) {
+  const int vel = g.nloc * g.NV;
+  if (mu >= vel) return true;
+  const int i = mu / g.NV;
+  return node_dead(g, 2 * cx + i % 3, 2 * cy + i / 3);
+}
+template <typename FT>
+__device__ inline void write_patch_projector(const Geom& g, int cx, int cy, FT* out, int tid, int nth) {
+  const int n = g.npatch;
+  for (int t = tid; t < n * n; t += nth) {
+    const int col = t / n, row = t - col * n;
+    out[t] = cvt<FT>((row == col && patch_entry_dead(g, cx, cy, row)) ? 1.f : 0.f);
+  }
+}
+
 inline long long patch_stride(int npatch) { return ((long long)npatch * npatch + 31) / 32 * 32; }
 
 // ------------------------------------------------------------------ errors

@@ -59,6 +59,13 @@ void invert_patches(const Geom& g, const int* rowptr, const double* vv, const do
                     const float* vv32, const float* vp32, const float* pv32, FT* jinv, int compute_f32, int* status,
                     void* scratch, int* flags, cudaStream_t st);
 
+// FP32 inverses of the patches of 60 unknowns and more (patch_inverse.cu), without pivoting: flags[p]
+// = 1 (the array is zeroed here) marks patches whose pivot fell below 1e-3, for which nothing is
+// written.  Returns false (nothing launched) for patch sizes it has no kernel for.
+template <typename FT>
+bool invert_panels(const Geom& g, const int* rowptr, const double* vv, const double* vp, const double* pv, FT* jinv,
+                   long long stride, int* flags, cudaStream_t st);
+
 // One colour phase of the smoother: y_K = J_K^{-1} R_K r for all cells of colour
 // `colour`; accumulate (averaged mode: z += y) or apply (coloured mode: z += omega y).
 // variant = 3 * column-batch index (4, 8, 16 columns in flight) + CTA-size index (128, 256, 512)

@@ -281,9 +281,9 @@ __global__ void diag_blocks(Geom g, TimeData td, AsmCoef cf, const double* __res
 // nodes, combined with the class constants, the time matrix T_ab and the factor
 // tau w_a, added into the BCSR blocks of the cell's node pairs.
 // WONLY = false: the part of the operator that does not depend on w (time coupling, viscous,
-// Nitsche terms, velocity-pressure blocks); w is not read.  WONLY = true: add the terms that
+// Nitsche terms, velocity-pressure blocks); w is not read.  WONLY = true (2D): add the terms that
 // depend on w (convection, Newton) to the time-diagonal blocks of an operator that already
-// holds that part.
+// holds that part; assemble_w3d and assemble_w_q4 do so in 3D and for order 4.
 // index of the unordered pair {a, b} of 1D Q2 nodes: (0,0) 0, (0,1) 1, (0,2) 2, (1,1) 3, (1,2) 4, (2,2) 5
 __device__ __forceinline__ int pair3(int a, int b) {
   const int lo = a < b ? a : b, hi = a < b ? b : a;
@@ -300,7 +300,8 @@ __global__ void __launch_bounds__(256) assemble_cells(Geom g, int colour, TimeDa
   constexpr int NL = NQ;
   constexpr int ND = NL * DIM;
   constexpr int NTMAX = DIM == 2 ? 5 : 3;
-  constexpr int NTC = DIM == 2 ? NTMAX : 1;  // precomputed convection/Newton matrices in 2D only
+  constexpr int NTC = DIM == 2 ? NTMAX : 1;  // convection/Newton matrices (2D)
+  static_assert(DIM == 2 || !WONLY, "3D has a kernel of its own for the part that depends on w");
   __shared__ double phi[NQ][NL];
   __shared__ double dphi[NQ][NL][DIM];
   __shared__ double qwd[NQ];
@@ -427,7 +428,7 @@ __global__ void __launch_bounds__(256) assemble_cells(Geom g, int colour, TimeDa
       __syncthreads();
     }
 
-    if (DIM == 2) {
+    {
       // time-diagonal entries only: (i, j, a, c, e)
       const int nd = NL * NL * nt * DIM * DIM;
       for (int t = threadIdx.x; t < nd; t += blockDim.x) {
@@ -437,34 +438,6 @@ __global__ void __launch_bounds__(256) assemble_cells(Geom g, int colour, TimeDa
         if (c == e) val += cm[a % NTC][i][j];
         const int r = a * DIM + c, sc = a * DIM + e;
         vv[(long long)slots[i * NL + j] * NV * NV + (long long)r * NV + sc] += val;
-      }
-    } else {
-      // one task per (i, j, a): the convection value and the d x d Newton block over the
-      // quadrature points, then the d x d entries of block (a, a) of node pair (i, j)
-      for (int t = threadIdx.x; t < NL * NL * nt; t += blockDim.x) {
-        const int a = t % nt, j = (t / nt) % NL, i = t / (nt * NL);
-        double conv = 0.0, newt[DIM][DIM];
-        for (int c = 0; c < DIM; ++c)
-          for (int e = 0; e < DIM; ++e) newt[c][e] = 0.0;
-        for (int q = 0; q < NQ; ++q) {
-          double u = 0.0;
-          for (int f = 0; f < DIM; ++f) u += wq[a][q][f] * dphi[q][j][f];
-          const double wpi = qwd[q] * phi[q][i];
-          conv += wpi * u;
-          if (cf.newton) {
-            const double pp = wpi * phi[q][j];
-            for (int c = 0; c < DIM; ++c)
-              for (int e = 0; e < DIM; ++e) newt[c][e] += pp * gw[a][q][c][e];
-          }
-        }
-        const double sa = cf.tau * td.w[a];
-        double* blk = vv + (long long)slots[i * NL + j] * NV * NV;
-        for (int c = 0; c < DIM; ++c)
-          for (int e = 0; e < DIM; ++e) {
-            double val = cf.newton ? newt[c][e] : 0.0;
-            if (c == e) val += conv;
-            blk[(long long)(a * DIM + c) * NV + a * DIM + e] += sa * val;
-          }
       }
     }
     return;
@@ -500,6 +473,232 @@ __global__ void __launch_bounds__(256) assemble_cells(Geom g, int colour, TimeDa
   }
 }
 
+
+// The part that depends on w in 3D (convection, Newton), added to the time-diagonal blocks: sum
+// factorisation over the tensor-product basis phi_i(q) = L_i1(q1) L_i2(q2) L_i3(q3) and the 3^3 Gauss
+// rule, like the 2D form in assemble_cells.  With p_d the unordered pair of 1D nodes (i_d, j_d),
+//   Newton (phi_j d_e w_c, phi_i) = sum_q1 W L L(p1) sum_q2 W L L(p2) sum_q3 W L L(p3) d_e w_c(q)
+// depends on (p1, p2, p3) only (6^3 values per (c, e)), and the convection (w . grad phi_j, phi_i) is
+// the sum of three such contractions of w_x, w_y, w_z in which direction d carries W L_i D_j instead.
+// About 17 000 FP64 FMAs per cell and Radau node where the quadrature per node pair took 275 000; the
+// read-modify-write of 729 d x d blocks is then the larger part.
+__global__ void __launch_bounds__(256) assemble_w3d(Geom g, int colour, TimeData td, AsmCoef cf,
+                                                   const double* __restrict__ w, const int* __restrict__ rowptr,
+                                                   double* __restrict__ vv) {
+  constexpr int NL = 27;
+  __shared__ double ll[3][3][6];     // W L_a L_b (q), direction, Gauss point, pair (a, b)
+  __shared__ double ld[3][3][9];     // W L_a d_b (q), physical derivative
+  __shared__ double wn[3][NL];       // w_a at the cell's nodes
+  __shared__ double sx[2][3][9][3];  // [L or D along x][c][node line (y, z)][q1]
+  __shared__ double sy[3][3][3][9];  // [LL, DL, LD along (x, y)][c][node z][q1 + 3 q2]
+  __shared__ double wq[3][NL];       // w_c at the Gauss points
+  __shared__ double gw[9][NL];       // d_e w_c, index 3 c + e
+  __shared__ double t2[12][3][36];   // two directions contracted (fields: 9 gradients, w_x, w_y, w_z)
+  __shared__ double nw[9][216];      // Newton blocks, pairs (p1, p2, p3)
+  __shared__ double cv[3][9][36];    // convection: direction d's (i_d, j_d), the other two pairs
+  __shared__ int base[NL], wx[NL], wy[NL];
+  double(*t1)[9][6] = reinterpret_cast<double(*)[9][6]>(&nw[0][0]);  // one direction contracted; dead before nw
+  const int tid = threadIdx.x, nt = g.nt, NV = g.NV;
+  int cx, cy, cz;
+  patch_cell(g, g.coff[colour] + blockIdx.x, cx, cy, cz);
+  for (int t = tid; t < 54; t += 256) {
+    const int d = t / 18, q = (t / 6) % 3, pr = t % 6;
+    const int pa = pr < 3 ? 0 : (pr < 5 ? 1 : 2), pb = pr < 3 ? pr : (pr < 5 ? pr - 2 : 2);  // inverse of pair3
+    ll[d][q][pr] = c_GW[q] * g.h[d] / 2.0 * c_L1[q][pa] * c_L1[q][pb];
+  }
+  for (int t = tid; t < 81; t += 256) {
+    const int d = t / 27, q = (t / 9) % 3, a = (t / 3) % 3, b = t % 3;
+    ld[d][q][a * 3 + b] = c_GW[q] * g.h[d] / 2.0 * c_L1[q][a] * (2.0 / g.h[d] * c_D1[q][b]);
+  }
+  // node (x, y, z) of the cell is column ((z wy + y) wx + x) of its row's slots from base on
+  for (int i = tid; i < NL; i += 256) {
+    const int ix = 2 * cx + i % 3, iy = 2 * cy + (i / 3) % 3, iz = 2 * cz + i / 9;
+    int lo, hi;
+    stencil_range(ix, g.nn[0], lo, hi);
+    wx[i] = hi - lo + 1;
+    stencil_range(iy, g.nn[1], lo, hi);
+    wy[i] = hi - lo + 1;
+    base[i] = (int)bcsr_slot(g, rowptr, ix, iy, iz, 2 * cx, 2 * cy, 2 * cz);
+  }
+  const int nf0 = cf.newton ? 0 : 9;  // without Newton's term the gradients of w are not needed
+  for (int a = 0; a < nt; ++a) {
+    __syncthreads();
+    for (int t = tid; t < 3 * NL; t += 256) {
+      const int i = t / 3, c = t % 3;
+      wn[c][i] = w[node_id(g, 2 * cx + i % 3, 2 * cy + (i / 3) % 3, 2 * cz + i / 9) * NV + a * 3 + c];
+    }
+    __syncthreads();
+    // w and its gradient at the Gauss points, one direction at a time
+    for (int t = tid; t < 2 * 81; t += 256) {
+      const int k = t / 81, c = (t / 27) % 3, yz = (t / 3) % 9, q = t % 3;
+      double s = 0.0;
+      for (int l = 0; l < 3; ++l) s += (k ? 2.0 / g.h[0] * c_D1[q][l] : c_L1[q][l]) * wn[c][yz * 3 + l];
+      sx[k][c][yz][q] = s;
+    }
+    __syncthreads();
+    for (int t = tid; t < 3 * 81; t += 256) {
+      const int k = t / 81, c = (t / 27) % 3, z = (t / 9) % 3, q2 = (t / 3) % 3, q1 = t % 3;
+      double s = 0.0;
+      for (int l = 0; l < 3; ++l)
+        s += (k == 2 ? 2.0 / g.h[1] * c_D1[q2][l] : c_L1[q2][l]) * sx[k == 1 ? 1 : 0][c][z * 3 + l][q1];
+      sy[k][c][z][q1 + 3 * q2] = s;
+    }
+    __syncthreads();
+    for (int t = tid; t < 4 * 81; t += 256) {
+      const int k = t / 81, c = (t / 27) % 3, q3 = (t / 9) % 3, q12 = t % 9;  // k: value, d_x, d_y, d_z
+      double s = 0.0;
+      for (int l = 0; l < 3; ++l)
+        s += (k == 3 ? 2.0 / g.h[2] * c_D1[q3][l] : c_L1[q3][l]) * sy[k == 1 ? 1 : (k == 2 ? 2 : 0)][c][l][q12];
+      if (k == 0)
+        wq[c][q3 * 9 + q12] = s;
+      else
+        gw[3 * c + k - 1][q3 * 9 + q12] = s;
+    }
+    __syncthreads();
+    // first contraction: over q3 to t1[f][q1 + 3 q2][p3]; for w_z over q2 to [q1 + 3 q3][p2]
+    for (int t = tid; t < (12 - nf0) * 54; t += 256) {
+      const int f = nf0 + t / 54, r = (t / 6) % 9, pr = t % 6, q1 = r % 3, q = r / 3;
+      const double* fv = f < 9 ? gw[f] : wq[f - 9];
+      double s = 0.0;
+      for (int l = 0; l < 3; ++l)
+        s += f == 11 ? ll[1][l][pr] * fv[q1 + 3 * l + 9 * q] : ll[2][l][pr] * fv[q1 + 3 * q + 9 * l];
+      t1[f][r][pr] = s;
+    }
+    __syncthreads();
+    // second: over q2 to t2[f][q1][p2 6 + p3]; for w_y over q1 to [q2][p1 6 + p3]; for w_z over q1 to
+    // [q3][p1 6 + p2]
+    for (int t = tid; t < (12 - nf0) * 108; t += 256) {
+      const int f = nf0 + t / 108, q = (t / 36) % 3, pa = (t / 6) % 6, pb = t % 6;
+      double s = 0.0;
+      for (int l = 0; l < 3; ++l) s += f < 10 ? ll[1][l][pa] * t1[f][q + 3 * l][pb] : ll[0][l][pa] * t1[f][l + 3 * q][pb];
+      t2[f][q][pa * 6 + pb] = s;
+    }
+    __syncthreads();
+    if (cf.newton)
+      for (int t = tid; t < 9 * 216; t += 256) {
+        const int f = t / 216, p1 = (t / 36) % 6, r = t % 36;
+        double s = 0.0;
+        for (int l = 0; l < 3; ++l) s += ll[0][l][p1] * t2[f][l][r];
+        nw[f][p1 * 36 + r] = s;
+      }
+    for (int t = tid; t < 3 * 324; t += 256) {
+      const int d = t / 324, ij = (t / 36) % 9, r = t % 36;
+      double s = 0.0;
+      for (int l = 0; l < 3; ++l) s += ld[d][l][ij] * t2[9 + d][l][r];
+      cv[d][ij][r] = s;
+    }
+    __syncthreads();
+    const double sa = cf.tau * td.w[a];
+#pragma unroll 4
+    for (int t = tid; t < NL * NL * 9; t += 256) {
+      const int ce = t % 9, ij = t / 9, j = ij % NL, i = ij / NL, c = ce / 3, e = ce % 3;
+      if (c != e && !cf.newton) continue;
+      const int i1 = i % 3, i2 = (i / 3) % 3, i3 = i / 9, j1 = j % 3, j2 = (j / 3) % 3, j3 = j / 9;
+      const int p1 = pair3(i1, j1), p2 = pair3(i2, j2), p3 = pair3(i3, j3);
+      double val = cf.newton ? nw[ce][p1 * 36 + p2 * 6 + p3] : 0.0;
+      if (c == e)
+        val += cv[0][i1 * 3 + j1][p2 * 6 + p3] + cv[1][i2 * 3 + j2][p1 * 6 + p3] + cv[2][i3 * 3 + j3][p1 * 6 + p2];
+      const long long slot = base[i] + (j3 * wy[i] + j2) * wx[i] + j1;
+      vv[(slot * NV + a * 3 + c) * NV + a * 3 + e] += sa * val;
+    }
+  }
+}
+
+// The same for order 4 in 2D (Q4 basis, 5 x 5 Gauss rule, 15 unordered pairs of 1D nodes): about 11 000
+// FMAs per cell and Radau node where the quadrature per node pair took 140 000.
+__device__ __forceinline__ int pair5(int a, int b) {
+  const int lo = a < b ? a : b, hi = a < b ? b : a;
+  return lo * 5 - lo * (lo - 1) / 2 + hi - lo;
+}
+
+__global__ void __launch_bounds__(256) assemble_w_q4(Geom g, int colour, TimeData td, AsmCoef cf,
+                                                    const double* __restrict__ w, const int* __restrict__ rowptr,
+                                                    double* __restrict__ vv) {
+  constexpr int NL = 25;
+  __shared__ double ll[2][5][15], ld[2][5][25];
+  __shared__ double wn[2][NL];
+  __shared__ double sx[2][2][5][5];  // [L or D along x][c][node y][q1]
+  __shared__ double wq[2][NL], gw[4][NL];
+  __shared__ double t1[6][5][15];    // fields: 4 gradients and w_x contracted over q2, w_y over q1
+  __shared__ double nw[4][225], cv[2][25][15];
+  __shared__ int base[NL], wx[NL];
+  const int tid = threadIdx.x, nt = g.nt, NV = g.NV;
+  int cx, cy, cz;
+  patch_cell(g, g.coff[colour] + blockIdx.x, cx, cy, cz);
+  for (int t = tid; t < 2 * 5 * 25; t += 256) {
+    const int d = t / 125, q = (t / 25) % 5, a = (t / 5) % 5, b = t % 5;
+    const double wt = c_GW4[q] * g.h[d] / 2.0;
+    ld[d][q][a * 5 + b] = wt * c_L4[q][a] * (2.0 / g.h[d] * c_D4[q][b]);
+    if (a <= b) ll[d][q][pair5(a, b)] = wt * c_L4[q][a] * c_L4[q][b];
+  }
+  for (int i = tid; i < NL; i += 256) {
+    const int ix = 4 * cx + i % 5, iy = 4 * cy + i / 5;
+    int lo, hi;
+    stencil_range(ix, g.nn[0], lo, hi, 4);
+    wx[i] = hi - lo + 1;
+    base[i] = (int)bcsr_slot(g, rowptr, ix, iy, 0, 4 * cx, 4 * cy, 0);
+  }
+  const int nf0 = cf.newton ? 0 : 4;
+  for (int a = 0; a < nt; ++a) {
+    __syncthreads();
+    for (int t = tid; t < 2 * NL; t += 256) {
+      const int i = t / 2, c = t % 2;
+      wn[c][i] = w[node_id(g, 4 * cx + i % 5, 4 * cy + i / 5, 0) * NV + a * 2 + c];
+    }
+    __syncthreads();
+    for (int t = tid; t < 100; t += 256) {
+      const int k = t / 50, c = (t / 25) % 2, y = (t / 5) % 5, q = t % 5;
+      double s = 0.0;
+      for (int l = 0; l < 5; ++l) s += (k ? 2.0 / g.h[0] * c_D4[q][l] : c_L4[q][l]) * wn[c][y * 5 + l];
+      sx[k][c][y][q] = s;
+    }
+    __syncthreads();
+    for (int t = tid; t < 150; t += 256) {
+      const int k = t / 50, c = (t / 25) % 2, q2 = (t / 5) % 5, q1 = t % 5;  // k: value, d_x, d_y
+      double s = 0.0;
+      for (int l = 0; l < 5; ++l)
+        s += (k == 2 ? 2.0 / g.h[1] * c_D4[q2][l] : c_L4[q2][l]) * sx[k == 1 ? 1 : 0][c][l][q1];
+      if (k == 0)
+        wq[c][q1 + 5 * q2] = s;
+      else
+        gw[2 * c + k - 1][q1 + 5 * q2] = s;
+    }
+    __syncthreads();
+    for (int t = tid; t < (6 - nf0) * 75; t += 256) {
+      const int f = nf0 + t / 75, q = (t / 15) % 5, pr = t % 15;
+      const double* fv = f < 4 ? gw[f] : wq[f - 4];
+      double s = 0.0;
+      for (int l = 0; l < 5; ++l) s += f == 5 ? ll[0][l][pr] * fv[l + 5 * q] : ll[1][l][pr] * fv[q + 5 * l];
+      t1[f][q][pr] = s;
+    }
+    __syncthreads();
+    if (cf.newton)
+      for (int t = tid; t < 4 * 225; t += 256) {
+        const int f = t / 225, p1 = (t / 15) % 15, p2 = t % 15;
+        double s = 0.0;
+        for (int l = 0; l < 5; ++l) s += ll[0][l][p1] * t1[f][l][p2];
+        nw[f][p1 * 15 + p2] = s;
+      }
+    for (int t = tid; t < 2 * 375; t += 256) {
+      const int d = t / 375, ij = (t / 15) % 25, pr = t % 15;
+      double s = 0.0;
+      for (int l = 0; l < 5; ++l) s += ld[d][l][ij] * t1[4 + d][l][pr];
+      cv[d][ij][pr] = s;
+    }
+    __syncthreads();
+    const double sa = cf.tau * td.w[a];
+#pragma unroll 4
+    for (int t = tid; t < NL * NL * 4; t += 256) {
+      const int ce = t % 4, ij = t / 4, j = ij % NL, i = ij / NL, c = ce / 2, e = ce % 2;
+      if (c != e && !cf.newton) continue;
+      const int i1 = i % 5, i2 = i / 5, j1 = j % 5, j2 = j / 5, p1 = pair5(i1, j1), p2 = pair5(i2, j2);
+      double val = cf.newton ? nw[ce][p1 * 15 + p2] : 0.0;
+      if (c == e) val += cv[0][i1 * 5 + j1][p2] + cv[1][i2 * 5 + j2][p1];
+      const long long slot = base[i] + j2 * wx[i] + j1;
+      vv[(slot * NV + a * 2 + c) * NV + a * 2 + e] += sa * val;
+    }
+  }
+}
 
 // Data terms of the right-hand side of Eq. (2.2), one CTA per face class:
 //   NB[(i,c),(j,e)]: B_GammaD(phi_j e_e, (phi_i e_c, 0)) = -nu <phi_j, d_n phi_i> delta_ce
@@ -608,10 +807,10 @@ __global__ void __launch_bounds__(256) assemble_rhs(Geom g, int colour, TimeData
 }
 
 // ---------------------------------------------------------------- order 4 (2D), (Q4)^2 x P3disc
-// One CTA per cell: the whole element matrix of the space-time block (time coupling, viscous,
-// convection and Newton at w_a, the Nitsche terms of the cell's Dirichlet faces) by quadrature
-// with the 5 x 5 Gauss rule (5 points per face), added into the cell's BCSR blocks, and the
-// velocity-pressure / pressure-velocity blocks.  w = nullptr: the operator at w = 0.
+// One CTA per cell: the part of the space-time element matrix that does not depend on w (time
+// coupling, viscous terms, the Nitsche terms of the cell's Dirichlet faces) by quadrature with the
+// 5 x 5 Gauss rule (5 points per face), added into the cell's BCSR blocks, and the
+// velocity-pressure / pressure-velocity blocks.
 // P3 monomials xi^a eta^b in the order (0,0) (1,0) (0,1) (2,0) (1,1) (0,2) (3,0) (2,1) (1,2) (0,3).
 __device__ __forceinline__ double p3_monomial(int m, double x, double y) {
   const int ea[10] = {0, 1, 0, 2, 1, 0, 3, 2, 1, 0}, eb[10] = {0, 0, 1, 0, 1, 2, 0, 1, 2, 3};
@@ -622,15 +821,12 @@ __device__ __forceinline__ double p3_monomial(int m, double x, double y) {
 }
 
 __global__ void __launch_bounds__(256) assemble_cells_q4(Geom g, int colour, TimeData td, AsmCoef cf,
-                                                         const double* __restrict__ w,
                                                          const int* __restrict__ rowptr, double* __restrict__ vv,
                                                          double* __restrict__ vp, double* __restrict__ pv) {
   constexpr int NL = 25, NQ = 25, NF = 5, NPD = 10;
   __shared__ double phi[NQ][NL];
   __shared__ double dphi[NQ][NL][2];
   __shared__ double qwd[NQ];
-  __shared__ double wq[5][NQ][2];
-  __shared__ double gw[5][NQ][2][2];
   __shared__ int slots[NL * NL];
   const int nt = g.nt, NV = g.NV;
   int cx, cy, cz;
@@ -652,37 +848,14 @@ __global__ void __launch_bounds__(256) assemble_cells_q4(Geom g, int colour, Tim
     slots[t] = (int)bcsr_slot(g, rowptr, 4 * cx + i % 5, 4 * cy + i / 5, 0, 4 * cx + j % 5, 4 * cy + j / 5, 0);
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < nt * NQ * 2; t += blockDim.x) {
-    const int a = t / (NQ * 2), q = (t / 2) % NQ, c = t % 2;
-    double v = 0.0, g0 = 0.0, g1 = 0.0;
-    if (w)
-      for (int i = 0; i < NL; ++i) {
-        const double wi = w[node_id(g, 4 * cx + i % 5, 4 * cy + i / 5, 0) * NV + a * 2 + c];
-        v += phi[q][i] * wi;
-        g0 += dphi[q][i][0] * wi;
-        g1 += dphi[q][i][1] * wi;
-      }
-    wq[a][q][c] = v;
-    gw[a][q][c][0] = g0;
-    gw[a][q][c][1] = g1;
-  }
-  __syncthreads();
-  // one task per node pair (i, j): the scalar integrals, the Newton and Nitsche d x d blocks
+  // one task per node pair (i, j): the scalar integrals and the Nitsche d x d block
   for (int t = threadIdx.x; t < NL * NL; t += blockDim.x) {
     const int i = t / NL, j = t % NL;
-    double mass = 0.0, stiff = 0.0, conv[5] = {0, 0, 0, 0, 0}, newt[5][2][2] = {};
+    double mass = 0.0, stiff = 0.0;
     for (int q = 0; q < NQ; ++q) {
       const double wpi = qwd[q] * phi[q][i];
       mass += wpi * phi[q][j];
       stiff += qwd[q] * (dphi[q][i][0] * dphi[q][j][0] + dphi[q][i][1] * dphi[q][j][1]);
-      for (int a = 0; a < nt; ++a) {
-        conv[a] += wpi * (wq[a][q][0] * dphi[q][j][0] + wq[a][q][1] * dphi[q][j][1]);
-        if (cf.newton) {
-          const double pp = wpi * phi[q][j];
-          for (int c = 0; c < 2; ++c)
-            for (int e = 0; e < 2; ++e) newt[a][c][e] += pp * gw[a][q][c][e];
-        }
-      }
     }
     double fs = 0.0, fn[2][2] = {{0, 0}, {0, 0}};
     for (int f = 0; f < 4; ++f) {
@@ -708,16 +881,14 @@ __global__ void __launch_bounds__(256) assemble_cells_q4(Geom g, int colour, Tim
           for (int e = 0; e < 2; ++e) {
             double val = c == e ? td.T[a][b] * mass : 0.0;
             if (a == b) {
-              double sp = fn[c][e] + (cf.newton ? newt[a][c][e] : 0.0);
-              if (c == e) sp += conv[a] + cf.nu * stiff + fs;
+              double sp = fn[c][e];
+              if (c == e) sp += cf.nu * stiff + fs;
               val += cf.tau * td.w[a] * sp;
             }
             blk[(long long)(a * 2 + c) * NV + b * 2 + e] += val;
           }
   }
-  // velocity-pressure [cell][i][a][c][m] and pressure-velocity [cell][a][m][i][c] (w-independent:
-  // written by the set-up's call, skipped by re-linearisations, vp == nullptr)
-  if (!vp) return;
+  // velocity-pressure [cell][i][a][c][m] and pressure-velocity [cell][a][m][i][c]
   for (int t = threadIdx.x; t < NL * 2 * NPD; t += blockDim.x) {
     const int m = t % NPD, c = (t / NPD) % 2, i = t / (NPD * 2);
     double val = 0.0;
@@ -763,24 +934,18 @@ long long assemble_table_doubles(int dim, int k) {
   return base + (long long)(k + 1) * (1LL << (2 * dim)) * nd * nd;  // followed by K
 }
 
-static void assemble_level_q4(const Geom& g, const TimeData& td, const AsmCoef& cf, const double* w_int,
-                              const int* rowptr, double* vv, long long nnzb, double* vp, double* pv, cudaStream_t st) {
-  STG_CUDA_OK(cudaMemsetAsync(vv, 0, sizeof(double) * nnzb * g.NV * g.NV, st));
-  for (int col = 0; col < 4; ++col) {
-    const long long cnt = g.coff[col + 1] - g.coff[col];
-    if (cnt == 0) continue;
-    assemble_cells_q4<<<(unsigned)cnt, 256, 0, st>>>(g, col, td, cf, w_int, rowptr, vv, vp, pv);
-    STG_LAUNCH_OK();
-  }
-}
-
 void assemble_level(const Geom& g, const TimeData& td, const AsmCoef& cf, const double* w_int, const int* rowptr,
                     double* tab, double* vv, long long nnzb, double* vp, double* pv, cudaStream_t st) {
-  if (g.r == 4) {  // order 4: the whole operator at w_int (null: w = 0) by the generic kernel
-    assemble_level_q4(g, td, cf, w_int, rowptr, vv, nnzb, vp, pv, st);
+  STG_CUDA_OK(cudaMemsetAsync(vv, 0, sizeof(double) * nnzb * g.NV * g.NV, st));
+  if (g.r == 4) {
+    for (int col = 0; col < 4; ++col) {
+      const long long cnt = g.coff[col + 1] - g.coff[col];
+      if (cnt == 0) continue;
+      assemble_cells_q4<<<(unsigned)cnt, 256, 0, st>>>(g, col, td, cf, rowptr, vv, vp, pv);
+      STG_LAUNCH_OK();
+    }
     return;
   }
-  STG_CUDA_OK(cudaMemsetAsync(vv, 0, sizeof(double) * nnzb * g.NV * g.NV, st));
   const unsigned ncls = 1u << (2 * g.dim);
   const int nloc = g.dim == 2 ? 9 : 27;
   double* K = tab + assemble_table_doubles(g.dim, -1);
@@ -812,21 +977,18 @@ void assemble_level(const Geom& g, const TimeData& td, const AsmCoef& cf, const 
 
 void assemble_level_w(const Geom& g, const TimeData& td, const AsmCoef& cf, const double* w_int, const int* rowptr,
                       const double* tab, const double* vconst, double* vv, long long nnzb, cudaStream_t st) {
-  if (g.r == 4) {
-    assemble_level_q4(g, td, cf, w_int, rowptr, vv, nnzb, nullptr, nullptr, st);
-    return;
-  }
   STG_CUDA_OK(cudaMemcpyAsync(vv, vconst, sizeof(double) * nnzb * g.NV * g.NV, cudaMemcpyDeviceToDevice, st));
   const double* K = tab + assemble_table_doubles(g.dim, -1);
   for (int col = 0; col < (1 << g.dim); ++col) {
     const long long cnt = g.coff[col + 1] - g.coff[col];
     if (cnt == 0) continue;
-    if (g.dim == 2)
+    if (g.r == 4)
+      assemble_w_q4<<<(unsigned)cnt, 256, 0, st>>>(g, col, td, cf, w_int, rowptr, vv);
+    else if (g.dim == 2)
       assemble_cells<2, true><<<(unsigned)cnt, 128, 0, st>>>(g, col, td, cf, w_int, rowptr, tab, K, vv, nullptr,
                                                            nullptr);
     else
-      assemble_cells<3, true><<<(unsigned)cnt, 256, 0, st>>>(g, col, td, cf, w_int, rowptr, tab, K, vv, nullptr,
-                                                           nullptr);
+      assemble_w3d<<<(unsigned)cnt, 256, 0, st>>>(g, col, td, cf, w_int, rowptr, vv);
     STG_LAUNCH_OK();
   }
 }

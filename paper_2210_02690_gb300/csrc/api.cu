@@ -190,6 +190,8 @@ struct LevelBufs {
   float *vv32 = nullptr, *vp32 = nullptr, *pv32 = nullptr;
   double* vconst = nullptr;  // the w = 0 assembly (time coupling, viscous, Nitsche), built once
   float *mk32 = nullptr, *ak32 = nullptr;  // Kronecker-split FP32 velocity rows (F32 form, levels >= 1, 2D)
+  float* w32 = nullptr;  // w and coefficients of the matrix-free FP32 residual (F32 form, levels >= 1, 3D and order 4)
+  void* mf = nullptr;
   void* jinv = nullptr;
   double* w = nullptr;
   double* asm_tab = nullptr;
@@ -221,6 +223,7 @@ struct stg_ctx {
   // the same for the intermediate levels, which are inverted concurrently with the finest
   void* inv_scratch2 = nullptr;
   int* inv_flags2 = nullptr;
+  float* mf_scr = nullptr;  // scratch of the matrix-free residual
   // FGMRES (finest level, internal layout, FP64)
   double *V = nullptr, *Z = nullptr, *wv = nullptr, *rv = nullptr, *partial = nullptr, *hd = nullptr;
   double *vin = nullptr, *vout = nullptr, *tmp_a = nullptr, *tmp_b = nullptr;
@@ -295,6 +298,19 @@ bool vc64(const stg_ctx* c) { return c->opt.vcycle_prec == STG_F64; }
 // FP64 coarse factors: always with the FP64 V-cycle, on request with the FP32 one
 bool coarse64(const stg_ctx* c) { return vc64(c) || c->opt.coarse_prec == STG_F64; }
 
+// The part of every level's operator that does not depend on w, and the coefficients of the matrix-free
+// residual.
+void assemble_constant(stg_ctx* c) {
+  const AsmCoef cf0{c->nu, c->tau, c->opt.gamma1, c->opt.gamma2, 0};
+  const AsmCoef cf{c->nu, c->tau, c->opt.gamma1, c->opt.gamma2, c->opt.linearisation == STG_NEWTON ? 1 : 0};
+  for (LevelBufs& L : c->lv) {
+    assemble_level(L.g, c->td, cf0, nullptr, L.rowptr, L.asm_tab, L.vv, L.nnzb, L.vp, L.pv, c->st);
+    STG_CUDA_OK(cudaMemcpyAsync(L.vconst, L.vv, sizeof(double) * L.nnzb * L.g.NV * L.g.NV,
+                                cudaMemcpyDeviceToDevice, c->st));
+    if (L.mf) residual_coef(L.g, c->td, cf, L.mf, c->st);
+  }
+}
+
 // Assemble every level for the finest-level linearisation velocity in F.w (internal
 // layout), invert the local matrices, factor the coarse system.
 void linearise_internal(stg_ctx* c) {
@@ -309,9 +325,11 @@ void linearise_internal(stg_ctx* c) {
   STG_CUDA_OK(cudaEventRecord(c->fork, c->st));
   STG_CUDA_OK(cudaStreamWaitEvent(c->side, c->fork, 0));
   STG_CUDA_OK(cudaStreamWaitEvent(c->aux, c->fork, 0));
-  // FP32 copies of a level's operator for the FP32 V-cycle (Kronecker split where there is one)
+  // what the FP32 V-cycle's residual needs of a level: w, or FP32 copies of the operator (Kronecker split
+  // where there is one)
   auto to_f32 = [&](LevelBufs& L, cudaStream_t s) {
-    if (vc64(c)) return;
+    if (L.w32) convert(L.g.nvel, L.w, L.w32, s);
+    if (!L.vp32) return;
     if (L.vv32) convert(L.nnzb * L.g.NV * L.g.NV, L.vv, L.vv32, s);
     const long long nvp = L.g.n_cells * L.g.nloc * L.g.nt * L.g.dim * L.g.npd;
     convert(nvp, L.vp, L.vp32, s);
@@ -394,7 +412,9 @@ void record_event(cudaEvent_t ev, cudaStream_t st) {
 
 template <typename VT>
 void residual(stg_ctx* c, const LevelBufs& L, const VT* x, const VT* b, VT* r) {
-  if (std::is_same<VT, float>::value && L.mk32)
+  if (std::is_same<VT, float>::value && L.mf)
+    residual_mf(L.g, L.mf, L.w32, (const float*)x, (const float*)b, c->mf_scr, (float*)r, c->st);
+  else if (std::is_same<VT, float>::value && L.mk32)
     apply_operator_kron(L.g, c->td, L.mk32, L.ak32, L.vp32, L.pv32, (const float*)x, (const float*)b,
                         (float*)r, c->st);
   else
@@ -950,10 +970,13 @@ stg_status stg_setup(const stg_mesh* mesh, int k, double nu, double tau, const d
       const long long nvp = g.n_cells * g.nloc * g.nt * g.dim * g.npd;
       L.vp = dalloc<double>(c, nvp);
       L.pv = dalloc<double>(c, nvp);
-      if (!f64) {
+      if (!f64 && l > 0 && residual_mf_supported(g)) {
+        L.w32 = dalloc<float>(c, g.nvel);
+        L.mf = dalloc<char>(c, (long long)residual_coef_bytes());
+      } else if (!f64 && l > 0) {
         L.vp32 = dalloc<float>(c, nvp);
         L.pv32 = dalloc<float>(c, nvp);
-        if (l > 0 && kron_supported(g)) {
+        if (kron_supported(g)) {
           // the FP32 residual takes the Kronecker form, and the patch inversion rounds the
           // FP64 blocks as it gathers them: no FP32 copy of the dense blocks
           L.mk32 = dalloc<float>(c, L.nnzb);
@@ -982,6 +1005,7 @@ stg_status stg_setup(const stg_mesh* mesh, int k, double nu, double tau, const d
     }
     if (scratch) c->inv_scratch = dalloc<char>(c, (long long)scratch);
     if (scratch2) c->inv_scratch2 = dalloc<char>(c, (long long)scratch2);
+    if (c->lv.back().mf) c->mf_scr = dalloc<float>(c, residual_scratch(c->lv.back().g));
     c->inv_flags = dalloc<int>(c, c->lv.back().g.n_cells);
     if (mesh->n_levels > 2) c->inv_flags2 = dalloc<int>(c, c->lv[mesh->n_levels - 2].g.n_cells);
     if (f64 || opt->coarse_prec == STG_F64)
@@ -1016,14 +1040,7 @@ stg_status stg_setup(const stg_mesh* mesh, int k, double nu, double tau, const d
     STG_CUDA_OK(cudaMallocHost(&c->hh, sizeof(double) * 160));
     // the part of every level's operator that does not depend on w: assembled once, together
     // with the element tables and the velocity-pressure blocks
-    {
-      const AsmCoef cf0{nu, tau, c->opt.gamma1, c->opt.gamma2, 0};
-      for (LevelBufs& L : c->lv) {
-        assemble_level(L.g, c->td, cf0, nullptr, L.rowptr, L.asm_tab, L.vv, L.nnzb, L.vp, L.pv, c->st);
-        STG_CUDA_OK(cudaMemcpyAsync(L.vconst, L.vv, sizeof(double) * L.nnzb * L.g.NV * L.g.NV,
-                                    cudaMemcpyDeviceToDevice, c->st));
-      }
-    }
+    assemble_constant(c);
     linearise(c, w);
     *out = c;
     return STG_OK;
@@ -1075,12 +1092,7 @@ stg_status stg_set_slab_length(stg_ctx* c, double tau) {
     // w-independent part of every level is assembled again, then the levels are
     // re-linearised at the current w (the last one set or left by the Newton iteration)
     c->tau = tau;
-    const AsmCoef cf0{c->nu, tau, c->opt.gamma1, c->opt.gamma2, 0};
-    for (LevelBufs& L : c->lv) {
-      assemble_level(L.g, c->td, cf0, nullptr, L.rowptr, L.asm_tab, L.vv, L.nnzb, L.vp, L.pv, c->st);
-      STG_CUDA_OK(cudaMemcpyAsync(L.vconst, L.vv, sizeof(double) * L.nnzb * L.g.NV * L.g.NV,
-                                  cudaMemcpyDeviceToDevice, c->st));
-    }
+    assemble_constant(c);
     linearise_internal(c);
     return STG_OK;
   } catch (const Error& e) {

@@ -50,6 +50,16 @@ template <typename MT, typename VT>
 void apply_operator(const Geom& g, const int* rowptr, const int* colidx, const MT* vv, const MT* vp, const MT* pv,
                     const VT* x, const VT* b, VT* out, cudaStream_t st);
 
+// The same in FP32 without a matrix (residual.cu), from the linearisation velocity w (FP32, internal
+// layout) and the coefficients that residual_coef writes to residual_coef_bytes() of device memory.
+// scratch: residual_scratch(g) floats.
+bool residual_mf_supported(const Geom& g);
+long long residual_scratch(const Geom& g);
+size_t residual_coef_bytes();
+void residual_coef(const Geom& g, const TimeData& td, const AsmCoef& cf, void* dst, cudaStream_t st);
+void residual_mf(const Geom& g, const void* coef, const float* w, const float* x, const float* b, float* scratch,
+                 float* out, cudaStream_t st);
+
 // Local inverses J_K^{-1} of every cell (gather from the assembled J, Gauss-Jordan
 // with partial pivoting in CT precision, stored as FT). status[0] receives the
 // first singular cell + 1 (0 = none).

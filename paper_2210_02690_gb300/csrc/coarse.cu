@@ -31,388 +31,88 @@ namespace stg {
 namespace {
 
 // ---------------------------------------------------------------- batched dense kernels
-// In-place Gauss-Jordan inverse with partial pivoting; one CTA per matrix.  With
-// SMEM the matrix is copied into shared memory first (when it fits).  Each
-// pivot step has three phases separated by barriers: pivot search (one warp);
-// row interchange, saved pivot column and scaled pivot row (all threads, from
-// the values before the interchange); rank-one update of the other rows.
-template <typename T, bool SMEM>
-__global__ void __launch_bounds__(1024) bgj_kernel(int m, T* const* As, int* status) {
-  T* G = As[blockIdx.x];
-  extern __shared__ __align__(16) unsigned char sh_raw[];
-  T* A = SMEM ? reinterpret_cast<T*>(sh_raw) : G;
-  T* colj = SMEM ? A + (long long)m * m : reinterpret_cast<T*>(sh_raw);
-  int* perm = reinterpret_cast<int*>(colj + m);
-  __shared__ int s_piv, s_fail;
-  __shared__ T s_pval, s_ajj;
-  const int tid = threadIdx.x, nth = blockDim.x;
-  const int w = tid >> 5, ln = tid & 31, nw = nth >> 5;
-  if (tid == 0) s_fail = 0;
-  if (SMEM)
-    for (long long t = tid; t < (long long)m * m; t += nth) A[t] = G[t];
-  __syncthreads();
-  for (int j = 0; j < m; ++j) {
-    if (tid < 32) {
-      T best = -1;
-      int bi = m;
-      for (int i = j + tid; i < m; i += 32) {
-        const T v = fabs(A[(long long)i * m + j]);
-        if (v > best || (v == best && i < bi)) {
-          best = v;
-          bi = i;
-        }
-      }
-      for (int off = 16; off > 0; off >>= 1) {
-        const T ob = __shfl_down_sync(0xffffffffu, best, off);
-        const int oi = __shfl_down_sync(0xffffffffu, bi, off);
-        if (ob > best || (ob == best && oi < bi)) {
-          best = ob;
-          bi = oi;
-        }
-      }
-      if (tid == 0) {
-        s_piv = bi;
-        const T pv = bi < m ? A[(long long)bi * m + j] : (T)0;
-        s_pval = pv;
-        s_ajj = A[(long long)j * m + j];
-        if (!(fabs(pv) > (T)0) || isinf(pv)) s_fail = 1;
-        perm[j] = bi;
-      }
-    }
-    __syncthreads();
-    if (s_fail) break;
-    const int pr = s_piv;
-    const T inv = (T)1 / s_pval;
-    // column j of every row before the interchange (rows j and pr swap their entries)
-    for (int i = tid; i < m; i += nth)
-      colj[i] = i == j ? s_pval : (i == pr ? s_ajj : A[(long long)i * m + j]);
-    // interchange rows j and pr, scale the new pivot row
-    for (int l = tid; l < m; l += nth) {
-      const T vj = A[(long long)j * m + l], vp = A[(long long)pr * m + l];
-      A[(long long)j * m + l] = l == j ? inv : vp * inv;
-      if (pr != j) A[(long long)pr * m + l] = vj;
-    }
-    __syncthreads();
-    {
-      const T* rj = A + (long long)j * m;
-      for (int i = w; i < m; i += nw) {
-        if (i == j) continue;
-        const T f = colj[i];
-        T* ri = A + (long long)i * m;
-        for (int l = ln; l < m; l += 32) ri[l] = (l == j ? (T)0 : ri[l]) - f * rj[l];
-      }
-    }
-    __syncthreads();
-  }
-  if (s_fail) {
-    if (tid == 0) atomicCAS(status, 0, 1 + (int)blockIdx.x);
-    return;
-  }
-  for (int j = m - 1; j >= 0; --j) {
-    const int pj = perm[j];
-    if (pj != j)
-      for (int i = tid; i < m; i += nth) {
-        const T t = A[(long long)i * m + j];
-        A[(long long)i * m + j] = A[(long long)i * m + pj];
-        A[(long long)i * m + pj] = t;
-      }
-    __syncthreads();
-  }
-  if (SMEM)
-    for (long long t = tid; t < (long long)m * m; t += nth) G[t] = A[t];
-}
-
-// Gauss-Jordan for matrices too large for shared memory: each pivot step is two launches over
-// the whole batch, so the rank-one updates (O(m^2) per step) spread over all SMs instead of one
-// CTA per matrix.  Same operations and order as bgj_kernel (first maximal pivot, saved pivot
-// column, row interchange, scaled pivot row, update, columns swapped back at the end).
-template <typename T>
-__global__ void __launch_bounds__(256) gj_pivot_kernel(int m, int j, T* const* As, T* __restrict__ col,
-                                                       int* __restrict__ perm, int* __restrict__ fail) {
-  const int b = blockIdx.x, tid = threadIdx.x;
-  if (fail[b]) return;
-  T* A = As[b];
-  T* cj = col + (long long)b * m;
-  __shared__ T s_best[256];
-  __shared__ int s_idx[256];
-  __shared__ int s_pr, s_bad;
-  __shared__ T s_pv, s_ajj;
-  T best = -1;
-  int bi = m;
-  for (int i = j + tid; i < m; i += blockDim.x) {
-    const T v = fabs(A[(long long)i * m + j]);
-    if (v > best || (v == best && i < bi)) {
-      best = v;
-      bi = i;
-    }
-  }
-  s_best[tid] = best;
-  s_idx[tid] = bi;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (tid < w) {
-      const T ob = s_best[tid + w];
-      const int oi = s_idx[tid + w];
-      if (ob > s_best[tid] || (ob == s_best[tid] && oi < s_idx[tid])) {
-        s_best[tid] = ob;
-        s_idx[tid] = oi;
-      }
-    }
-    __syncthreads();
-  }
-  if (tid == 0) {
-    const int pr = s_idx[0];
-    const T pv = pr < m ? A[(long long)pr * m + j] : (T)0;
-    s_pr = pr;
-    s_pv = pv;
-    s_ajj = A[(long long)j * m + j];
-    s_bad = (!(fabs(pv) > (T)0) || isinf(pv)) ? 1 : 0;
-    if (s_bad) fail[b] = 1;
-    perm[(long long)b * m + j] = pr;
-  }
-  __syncthreads();
-  if (s_bad) return;
-  const int pr = s_pr;
-  const T inv = (T)1 / s_pv;
-  for (int i = tid; i < m; i += blockDim.x) cj[i] = i == j ? s_pv : (i == pr ? s_ajj : A[(long long)i * m + j]);
-  __syncthreads();
-  for (int l = tid; l < m; l += blockDim.x) {
-    const T vj = A[(long long)j * m + l], vp = A[(long long)pr * m + l];
-    A[(long long)j * m + l] = l == j ? inv : vp * inv;
-    if (pr != j) A[(long long)pr * m + l] = vj;
-  }
-}
-
-// A[i][l] = (l == j ? 0 : A[i][l]) - col[i] A[j][l] for all i != j; 32 columns x 32 rows a block
-template <typename T>
-__global__ void __launch_bounds__(256) gj_update_kernel(int m, int j, T* const* As, const T* __restrict__ col,
-                                                        const int* __restrict__ fail) {
-  const int b = blockIdx.z;
-  if (fail[b]) return;
-  T* A = As[b];
-  const T* cj = col + (long long)b * m;
-  const int l = blockIdx.x * 32 + (threadIdx.x & 31);
-  if (l >= m) return;
-  const T rj = A[(long long)j * m + l];
-  const int i0 = blockIdx.y * 32 + (threadIdx.x >> 5);
-  for (int r = 0; r < 4; ++r) {
-    const int i = i0 + 8 * r;
-    if (i >= m || i == j) continue;
-    T* ai = A + (long long)i * m + l;
-    *ai = (l == j ? (T)0 : *ai) - cj[i] * rj;
-  }
-}
-
-// Blocked Gauss-Jordan for the large blocks: the same pivots and operations as gj_pivot_kernel /
-// gj_update_kernel, arranged by panels of w columns [c0, c0 + w).  Within a panel every step
-// (first maximal pivot among the rows not yet used, row interchange, scaled pivot row, update)
-// runs on the m x w panel in shared memory; the other columns are updated once per panel:
-// with P the panel's pivot rows, Q the panel columns and C the others, w Gauss-Jordan steps turn
-// A_PC into A_PQ^{-1} A_PC and A_RC into A_RC - A_RQ A_PQ^{-1} A_PC, i.e.
-//   A[:, C] = [0 on rows P; A_RC] + panel_new A_PC_old,
-// one batched product (panel_new is the m x w panel after its steps: A_PQ^{-1} on rows P and
-// -A_RQ A_PQ^{-1} on the others).  3 launches per panel instead of 2 per column.
-template <typename T>
-__global__ void __launch_bounds__(1024) gjb_panel_kernel(int m, int c0, int w, T* const* As, T* const* Ps,
-                                                         int* __restrict__ perm, long long pstride,
-                                                         int* __restrict__ fail) {
-  const int b = blockIdx.x, tid = threadIdx.x, nth = blockDim.x;
-  if (fail[b]) return;
-  T* A = As[b];
-  extern __shared__ __align__(16) unsigned char sh_raw[];
-  const int ld = w + 1;  // padded row stride: a panel column read across rows spreads over the banks
-  T* P = reinterpret_cast<T*>(sh_raw);
-  T* colj = P + (long long)m * ld;
-  __shared__ T s_best[32];
-  __shared__ int s_idx[32];
-  __shared__ int s_pr, s_bad;
-  __shared__ T s_pv;
-  for (long long t = tid; t < (long long)m * w; t += nth) {
-    const int i = (int)(t / w), l = (int)(t - (long long)i * w);
-    P[i * ld + l] = A[(long long)i * m + c0 + l];
-  }
-  __syncthreads();
-  for (int jj = 0; jj < w; ++jj) {
-    const int j = c0 + jj;
-    T best = -1;
-    int bi = m;
-    for (int i = j + tid; i < m; i += nth) {
-      const T v = fabs(P[i * ld + jj]);
-      if (v > best || (v == best && i < bi)) {
-        best = v;
-        bi = i;
-      }
-    }
-    for (int off = 16; off > 0; off >>= 1) {
-      const T ob = __shfl_down_sync(0xffffffffu, best, off);
-      const int oi = __shfl_down_sync(0xffffffffu, bi, off);
-      if (ob > best || (ob == best && oi < bi)) {
-        best = ob;
-        bi = oi;
-      }
-    }
-    if ((tid & 31) == 0) {
-      s_best[tid >> 5] = best;
-      s_idx[tid >> 5] = bi;
-    }
-    __syncthreads();
-    if (tid < 32) {
-      best = tid < (nth >> 5) ? s_best[tid] : (T)-1;
-      bi = tid < (nth >> 5) ? s_idx[tid] : m;
-      for (int off = 16; off > 0; off >>= 1) {
-        const T ob = __shfl_down_sync(0xffffffffu, best, off);
-        const int oi = __shfl_down_sync(0xffffffffu, bi, off);
-        if (ob > best || (ob == best && oi < bi)) {
-          best = ob;
-          bi = oi;
-        }
-      }
-      if (tid == 0) {
-        const T pv = bi < m ? P[bi * ld + jj] : (T)0;
-        s_pr = bi;
-        s_pv = pv;
-        s_bad = (!(fabs(pv) > (T)0) || isinf(pv)) ? 1 : 0;
-        if (s_bad) fail[b] = 1;
-        perm[(long long)b * pstride + j] = bi;
-      }
-    }
-    __syncthreads();
-    if (s_bad) return;  // block-uniform; the matrix is reported by gj_unpermute_kernel
-    const int pr = s_pr;
-    if (pr != j)
-      for (int l = tid; l < w; l += nth) {
-        const T t = P[j * ld + l];
-        P[j * ld + l] = P[pr * ld + l];
-        P[pr * ld + l] = t;
-      }
-    __syncthreads();
-    const T inv = (T)1 / s_pv;
-    for (int i = tid; i < m; i += nth) colj[i] = P[i * ld + jj];
-    __syncthreads();
-    for (int l = tid; l < w; l += nth) P[j * ld + l] = (l == jj ? (T)1 : P[j * ld + l]) * inv;
-    __syncthreads();
-    for (long long t = tid; t < (long long)m * w; t += nth) {
-      const int i = (int)(t / w), l = (int)(t - (long long)i * w);
-      if (i == j) continue;
-      P[i * ld + l] = (l == jj ? (T)0 : P[i * ld + l]) - colj[i] * P[j * ld + l];
-    }
-    __syncthreads();
-  }
-  T* pn = Ps[b];
-  for (long long t = tid; t < (long long)m * w; t += nth) {
-    const int i = (int)(t / w), l = (int)(t - (long long)i * w);
-    const T v = P[i * ld + l];
-    A[(long long)i * m + c0 + l] = v;
-    pn[t] = v;
-  }
-}
-
-// The panel's row interchanges applied to the other columns (in order), then the pivot rows'
-// old values of the other columns saved (zero in the panel's own columns) and cleared in A.
-template <typename T>
-__global__ void __launch_bounds__(256) gjb_swap_save_kernel(int m, int c0, int w, T* const* As, T* const* Os,
-                                                            const int* __restrict__ perm, long long pstride,
-                                                            const int* __restrict__ fail) {
-  const int b = blockIdx.y;
-  if (fail[b]) return;
-  const int l = blockIdx.x * blockDim.x + threadIdx.x;
-  if (l >= m) return;
-  T* A = As[b];
-  T* O = Os[b];
-  const bool panel = l >= c0 && l < c0 + w;
-  if (!panel)
-    for (int t = 0; t < w; ++t) {
-      const int j = c0 + t, pr = perm[(long long)b * pstride + j];
-      if (pr != j) {
-        const T x = A[(long long)j * m + l];
-        A[(long long)j * m + l] = A[(long long)pr * m + l];
-        A[(long long)pr * m + l] = x;
-      }
-    }
-  for (int t = 0; t < w; ++t) {
-    T* a = A + (long long)(c0 + t) * m + l;
-    O[(long long)t * m + l] = panel ? (T)0 : *a;
-    if (!panel) *a = (T)0;
-  }
-}
-
-// columns swapped back (last interchange first); the status records the first failed matrix
-template <typename T>
-__global__ void __launch_bounds__(1024) gj_unpermute_kernel(int m, T* const* As, const int* __restrict__ perm,
-                                                            const int* __restrict__ fail, int* status) {
-  const int b = blockIdx.x;
-  if (fail[b]) {
-    if (threadIdx.x == 0) atomicCAS(status, 0, 1 + b);
-    return;
-  }
-  T* A = As[b];
-  const int* pm = perm + (long long)b * m;
-  for (int j = m - 1; j >= 0; --j) {
-    const int pj = pm[j];
-    if (pj != j)
-      for (int i = threadIdx.x; i < m; i += blockDim.x) {
-        const T t = A[(long long)i * m + j];
-        A[(long long)i * m + j] = A[(long long)i * m + pj];
-        A[(long long)i * m + pj] = t;
-      }
-    __syncthreads();
-  }
-}
-
 // C = alpha (A0 B0 + A1 B1) + beta C, batched through pointer arrays, row-major (A: M x K, B:
-// K x N, C: M x N); a null A0/A1 (per item) drops its product.  64 x 64 tiles, 16-deep k slices
-// staged in shared memory, 4 x 4 outputs per thread.
-template <typename T>
-__global__ void __launch_bounds__(256) bgemm2_kernel(int M, int N, int K, T alpha, const T* const* A0s,
-                                                     const T* const* B0s, const T* const* A1s,
-                                                     const T* const* B1s, T beta, T* const* Cs) {
-  constexpr int BM = 64, BN = 64, BK = 16;
-  __shared__ __align__(16) T sa[BK][BM + 4];
-  __shared__ __align__(16) T sb[BK][BN + 4];
-  const int b = blockIdx.z, tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
+// K x N, C: M x N); a null A0/A1 (per item) drops its product.  (TM TY) x (TN TX) tiles, TM x TN outputs a
+// thread, 16-deep k slices staged in shared memory, the next slice's loads in flight during a slice's FMAs.
+// A slice whose staged A or B is all zero is skipped: the couplings between planes and slabs (A_IV, A_VI)
+// are banded in the node lines, so a tile meets a third to a half of their k range.
+// Tiles: 48 x 48 for the blocks of 2D coarse levels (134 and 226 rows leave 7% and 6% of a 48-wide tiling empty,
+// 43% and 13% of a 64-wide one), 128 x 128 from 512 rows on (FP32).  FP64 is bound by GB300's FP64 pipe.
+template <typename T, int TM, int TN, int TX, int TY>
+__global__ void __launch_bounds__(TX* TY, TX * TY == 64 ? 8 : 2) bgemm2_kernel(int M, int N, int K, T alpha, const T* const* A0s,
+                                                       const T* const* B0s, const T* const* A1s, const T* const* B1s,
+                                                       T beta, T* const* Cs) {
+  constexpr int BM = TM * TY, BN = TN * TX, BK = 16, NTH = TX * TY;
+  constexpr int LA = (BM * BK + NTH - 1) / NTH, LB = (BN * BK + NTH - 1) / NTH;
+  constexpr int PAD = 16 / sizeof(T);
+  __shared__ __align__(16) T sa[BK][BM + PAD];
+  __shared__ __align__(16) T sb[BK][BN + PAD];
+  const int b = blockIdx.z, tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
   const int r0 = blockIdx.y * BM, c0 = blockIdx.x * BN;
-  T acc[4][4];
+  T acc[TM][TN];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0;
+    for (int j = 0; j < TN; ++j) acc[i][j] = 0;
   for (int pr = 0; pr < 2; ++pr) {
     const T* const* As = pr == 0 ? A0s : A1s;
     const T* const* Bs = pr == 0 ? B0s : B1s;
     const T* A = As ? As[b] : nullptr;
     if (!A) continue;  // the same for the whole CTA
     const T* B = Bs[b];
+    T ra[LA], rb[LB];
+    auto load = [&](int k0) {
+#pragma unroll
+      for (int u = 0; u < LA; ++u) {
+        const int t = tid + u * NTH, i = t / BK, k = k0 + t % BK, r = r0 + i;
+        ra[u] = (i < BM && r < M && k < K) ? A[(long long)r * K + k] : (T)0;
+      }
+#pragma unroll
+      for (int u = 0; u < LB; ++u) {
+        const int t = tid + u * NTH, kk = t / BN, k = k0 + kk, c = c0 + t % BN;
+        rb[u] = (kk < BK && k < K && c < N) ? B[(long long)k * N + c] : (T)0;
+      }
+    };
+    load(0);
     for (int k0 = 0; k0 < K; k0 += BK) {
-      for (int t = tid; t < BM * BK; t += 256) {
-        const int i = t / BK, kk = t % BK, r = r0 + i, k = k0 + kk;
-        sa[kk][i] = (r < M && k < K) ? A[(long long)r * K + k] : (T)0;
+      bool za = false, zb = false;
+#pragma unroll
+      for (int u = 0; u < LA; ++u) {
+        const int t = tid + u * NTH;
+        if (t / BK < BM) sa[t % BK][t / BK] = ra[u];
+        za |= ra[u] != (T)0;
       }
-      for (int t = tid; t < BK * BN; t += 256) {
-        const int kk = t / BN, j = t % BN, k = k0 + kk, c = c0 + j;
-        sb[kk][j] = (k < K && c < N) ? B[(long long)k * N + c] : (T)0;
+#pragma unroll
+      for (int u = 0; u < LB; ++u) {
+        const int t = tid + u * NTH;
+        if (t / BN < BK) sb[t / BN][t % BN] = rb[u];
+        zb |= rb[u] != (T)0;
       }
-      __syncthreads();
+      const bool any_a = __syncthreads_or(za), any_b = __syncthreads_or(zb);
+      if (k0 + BK < K) load(k0 + BK);
+      if (any_a && any_b) {
+#pragma unroll 4
+        for (int kk = 0; kk < BK; ++kk) {
+          T a[TM], bb[TN];
 #pragma unroll
-      for (int kk = 0; kk < BK; ++kk) {
-        T a[4], bb[4];
+          for (int i = 0; i < TM; ++i) a[i] = sa[kk][ty * TM + i];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = sa[kk][ty * 4 + i];
+          for (int j = 0; j < TN; ++j) bb[j] = sb[kk][tx * TN + j];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) bb[j] = sb[kk][tx * 4 + j];
+          for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] += a[i] * bb[j];
+            for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
+        }
       }
       __syncthreads();
     }
   }
   T* C = Cs[b];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int r = r0 + ty * 4 + i, c = c0 + tx * 4 + j;
+    for (int j = 0; j < TN; ++j) {
+      const int r = r0 + ty * TM + i, c = c0 + tx * TN + j;
       if (r < M && c < N) {
         T* p = C + (long long)r * N + c;
         *p = alpha * acc[i][j] + (beta == (T)0 ? (T)0 : beta * *p);
@@ -727,28 +427,23 @@ void CoarseSolver<T>::init(const Geom& geom, bool pure_dirichlet) {
   alloc(&GU, nsv * mV * mV);
   alloc(&bV, nsv * mV);
   {
+    // scratch of the Gauss-Jordan inverses: a second copy of every block of a batch, its panels, and
+    // the pivot rows
     const long long nb = std::max(nsi, nsv), mm = std::max(mI, mV);
-    alloc(&gj_scr, nb * mm);
-    STG_CUDA_OK(cudaMalloc(&gj_perm, sizeof(int) * nb * mm));
-    owned.push_back(gj_perm);
-    STG_CUDA_OK(cudaMalloc(&gj_fail, sizeof(int) * nb));
-    owned.push_back(gj_fail);
-    if (mm >= 512) {
-      // blocked Gauss-Jordan scratch: panels of at most 32 columns (FP32) or 16 (FP64)
-      gjb.w = sizeof(T) == 4 ? 32 : 16;
-      gjb.m_max = mm;
-      gjb.batch_max = (int)nb;
-      T *pan = nullptr, *old = nullptr;
-      alloc(&pan, nb * mm * gjb.w);
-      alloc(&old, nb * mm * gjb.w);
-      std::vector<T*> hp(nb), ho(nb);
-      for (long long b = 0; b < nb; ++b) {
-        hp[b] = pan + b * mm * gjb.w;
-        ho[b] = old + b * mm * gjb.w;
-      }
-      gjb.panels = upload_ptrs(hp, owned);
-      gjb.olds = upload_ptrs(ho, owned);
+    T *alt = nullptr, *pan = nullptr;
+    alloc(&alt, nb * mm * mm);
+    alloc(&pan, nb * gj_panel_values(mm));
+    std::vector<T*> ha(nb), hp(nb);
+    for (long long b = 0; b < nb; ++b) {
+      ha[b] = alt + b * mm * mm;
+      hp[b] = pan + b * gj_panel_values(mm);
     }
+    gj.alt = upload_ptrs(ha, owned);
+    gj.panel = upload_ptrs(hp, owned);
+    STG_CUDA_OK(cudaMalloc(&gj.piv, sizeof(int) * nb * (2 * mm + 1)));
+    owned.push_back(gj.piv);
+    gj.pos = gj.piv + nb * mm;
+    gj.fail = gj.pos + nb * mm;
   }
   alloc(&xV, nsv * mV);
   alloc(&bI, nsi * mI);
@@ -956,77 +651,21 @@ void CoarseSolver<T>::release() {
   owned.clear();
 }
 
-// Batched in-place inverses.  scratch: batch * m values of T, perm: batch * m ints, fail: batch
-// ints (used only for matrices of 512 rows or more, which take the multi-launch form).
-// FP32 blocks of up to 256 rows go to the on-chip Gauss-Jordan (coarse_gj.cu)
-static bool rgj(int m, float* const* A, int batch, int* status, cudaStream_t st) {
-  return rgj_invert(m, A, batch, status, st);
-}
-static bool rgj(int, double* const*, int, int*, cudaStream_t) { return false; }
-
-template <typename T>
-static void gemm2(int M, int N, int K, T alpha, const T* const* A0, const T* const* B0, const T* const* A1,
-                  const T* const* B1, T beta, T* const* C, int batch, cudaStream_t st);
-
-template <typename T>
-static void gj(int m, T* const* A, int batch, int* status, T* scratch, int* perm, int* fail, const GjBlocked& blk,
-               cudaStream_t st) {
-  if (batch <= 0 || m <= 0) return;
-  if (rgj(m, A, batch, status, st)) return;
-  const size_t tail = sizeof(T) * m + sizeof(int) * m;
-  const size_t full = sizeof(T) * (size_t)m * m + tail;
-  if (full <= 220 * 1024) {  // the whole matrix in shared memory
-    STG_CUDA_OK(cudaFuncSetAttribute(bgj_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)std::max<size_t>(full, 48 * 1024)));
-    bgj_kernel<T, true><<<batch, 1024, full, st>>>(m, A, status);
-    STG_LAUNCH_OK();
-    return;
-  }
-  if (m < 512) {  // one CTA per matrix in global memory: faster than 2m launches at this size
-    STG_CUDA_OK(cudaFuncSetAttribute(bgj_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)std::max<size_t>(tail, 48 * 1024)));
-    bgj_kernel<T, false><<<batch, 1024, tail, st>>>(m, A, status);
-    STG_LAUNCH_OK();
-    return;
-  }
-  STG_CUDA_OK(cudaMemsetAsync(fail, 0, sizeof(int) * batch, st));
-  if (blk.panels && blk.m_max >= m && blk.batch_max >= batch) {
-    // blocked form: panels of w columns in shared memory, one batched product per panel
-    int w = blk.w;
-    while (w > 4 && ((size_t)m * (w + 1) + m) * sizeof(T) > 200 * 1024) w /= 2;
-    const size_t sm = ((size_t)m * (w + 1) + m) * sizeof(T);
-    STG_CUDA_OK(cudaFuncSetAttribute(gjb_panel_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)std::max<size_t>(sm, 48 * 1024)));
-    const dim3 sgrid((m + 255) / 256, batch);
-    for (int c0 = 0; c0 < m; c0 += w) {
-      const int wp = std::min(w, m - c0);
-      gjb_panel_kernel<T><<<batch, 1024, sm, st>>>(m, c0, wp, A, (T* const*)blk.panels, perm, m, fail);
-      STG_LAUNCH_OK();
-      gjb_swap_save_kernel<T><<<sgrid, 256, 0, st>>>(m, c0, wp, A, (T* const*)blk.olds, perm, m, fail);
-      STG_LAUNCH_OK();
-      gemm2<T>(m, m, wp, (T)1, (const T* const*)blk.panels, (const T* const*)blk.olds, nullptr, nullptr, (T)1, A,
-               batch, st);
-    }
-  } else {
-    const dim3 ugrid((m + 31) / 32, (m + 31) / 32, batch);
-    for (int j = 0; j < m; ++j) {
-      gj_pivot_kernel<T><<<batch, 256, 0, st>>>(m, j, A, scratch, perm, fail);
-      STG_LAUNCH_OK();
-      gj_update_kernel<T><<<ugrid, 256, 0, st>>>(m, j, A, scratch, fail);
-      STG_LAUNCH_OK();
-    }
-  }
-  gj_unpermute_kernel<T><<<batch, 1024, 0, st>>>(m, A, perm, fail, status);
-  STG_LAUNCH_OK();
-}
-
 template <typename T>
 static void gemm2(int M, int N, int K, T alpha, const T* const* A0, const T* const* B0, const T* const* A1,
                   const T* const* B1, T beta, T* const* C, int batch, cudaStream_t st) {
   if (batch <= 0) return;
-  dim3 grid((N + 63) / 64, (M + 63) / 64, batch);
-  bgemm2_kernel<T><<<grid, 256, 0, st>>>(M, N, K, alpha, A0, B0, A1, B1, beta, C);
-  STG_LAUNCH_OK();
+  auto run = [&](auto kern, int bm, int bn, int threads) {
+    const dim3 grid((N + bn - 1) / bn, (M + bm - 1) / bm, batch);
+    kern<<<grid, threads, 0, st>>>(M, N, K, alpha, A0, B0, A1, B1, beta, C);
+    STG_LAUNCH_OK();
+  };
+  if constexpr (sizeof(T) == 8)
+    run(bgemm2_kernel<T, 3, 3, 16, 16>, 48, 48, 256);
+  else if (M >= 512 && N >= 512)
+    run(bgemm2_kernel<T, 8, 8, 16, 16>, 128, 128, 256);
+  else
+    run(bgemm2_kernel<T, 6, 6, 8, 8>, 48, 48, 64);
 }
 
 // One plan step as a launch of its own.
@@ -1066,7 +705,7 @@ void CoarseSolver<T>::factor(const int* rowptr, const int* colidx, const double*
     STG_LAUNCH_OK();
   }
   // interiors: A_II^{-1}, W = A_II^{-1} A_IV, C = A_VI W, S = A_VV - C (scattered)
-  gj<T>((int)mI, d_AII, (int)nsi, v.status, gj_scr, gj_perm, gj_fail, gjb, st);
+  gj_invert<T>((int)mI, d_AII, (int)nsi, v.status, gj, st);
   const T one = 1, zero = 0, mone = -1;
   gemm2<T>((int)mI, (int)(2 * mV), (int)mI, one, d_AII, d_AIV, nullptr, nullptr, zero, d_W, (int)nsi, st);
   gemm2<T>((int)(2 * mV), (int)(2 * mV), (int)mI, one, d_AVI, d_W, nullptr, nullptr, zero, d_C, (int)nsi, st);
@@ -1075,7 +714,7 @@ void CoarseSolver<T>::factor(const int* rowptr, const int* colidx, const double*
   // block cyclic reduction of the vertex-plane system
   const int m = (int)mV;
   for (const auto& lv : levels) {
-    gj<T>(m, lv.oD, lv.n_odd, v.status, gj_scr, gj_perm, gj_fail, gjb, st);
+    gj_invert<T>(m, lv.oD, lv.n_odd, v.status, gj, st);
     // [GL_i | GU_i] = D_i^{-1} [L_i | U_i]
     gemm2<T>(m, m, m, one, lv.gA, lv.gB, nullptr, nullptr, zero, lv.gC, 2 * lv.n_odd, st);
     // PL_j = L_j D_{j-st}^{-1}, PR_j = U_j D_{j+st}^{-1} (the solve's forward products)
@@ -1085,7 +724,7 @@ void CoarseSolver<T>::factor(const int* rowptr, const int* colidx, const double*
     // L_j <- -L_j GL_{j-st}, U_j <- -U_j GU_{j+st}, into new blocks
     gemm2<T>(m, m, m, mone, lv.uA, lv.uB, nullptr, nullptr, zero, lv.uC, lv.n_left + lv.n_right, st);
   }
-  gj<T>(m, d_top, 1, v.status, gj_scr, gj_perm, gj_fail, gjb, st);
+  gj_invert<T>(m, d_top, 1, v.status, gj, st);
 }
 
 template <typename T>

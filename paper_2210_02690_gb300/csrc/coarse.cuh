@@ -8,11 +8,19 @@
 
 namespace stg {
 
-// In-place inverses of `batch` FP32 m x m row-major matrices (m <= 256) by the on-chip
-// Gauss-Jordan kernel; status gets 1 + the first singular matrix.  Returns false (nothing
-// launched) for larger m.
-bool rgj_invert(int m, float* const* A, int batch, int* status, cudaStream_t st);
-
+// Scratch of gj_invert for batches of matrices of up to m_max rows: device arrays of pointers to one m_max x m_max
+// block and three m_max x 32 panels per matrix (panel values, multipliers, pivot rows; 32 reciprocal pivots behind),
+// and per matrix m_max pivot rows (piv), m_max row positions (pos) and a failure flag.
+template <typename T>
+struct GjScratch {
+  T **alt = nullptr, **panel = nullptr;
+  int *piv = nullptr, *pos = nullptr, *fail = nullptr;
+};
+inline long long gj_panel_values(long long m_max) { return 3 * 32 * m_max + 32; }
+// In-place inverses of `batch` m x m row-major matrices by Gauss-Jordan with partial pivoting;
+// status gets 1 + the index of a singular matrix (coarse_gj.cu).
+template <typename T>
+void gj_invert(int m, T* const* A, int batch, int* status, const GjScratch<T>& s, cudaStream_t st);
 
 template <typename T>
 struct CoarseView {
@@ -40,16 +48,6 @@ struct CrLevel {
   // (n_left + n_right items: A = uA, B = pB, C = pC)
   T **eA0, **eA1;
   T **gA, **gB, **gC, **dB0, **dB1, **dC, **uA, **uB, **uC, **pB, **pC;
-};
-
-// Scratch of the blocked Gauss-Jordan (blocks of 512+ rows): per matrix an m x w panel and a
-// w x m copy of the pivot rows, addressed through device pointer arrays.
-struct GjBlocked {
-  void* panels = nullptr;  // T** [batch_max]
-  void* olds = nullptr;    // T** [batch_max]
-  int w = 32;
-  long long m_max = 0;
-  int batch_max = 0;
 };
 
 // One step of the coarse solve (its plan is built once, at init), one launch each:
@@ -83,9 +81,7 @@ struct CoarseSolver {
   T **d_bI = nullptr, **d_gI = nullptr, **d_xVs = nullptr, **d_xI = nullptr;
   T **d_cA0 = nullptr, **d_cx0 = nullptr, **d_cA1 = nullptr, **d_cx1 = nullptr, **d_cy = nullptr;
   T **d_top = nullptr, **d_topb = nullptr, **d_topx = nullptr;
-  T* gj_scr = nullptr;  // Gauss-Jordan scratch for blocks too large for shared memory
-  int *gj_perm = nullptr, *gj_fail = nullptr;
-  GjBlocked gjb;
+  GjScratch<T> gj;
   std::vector<CrLevel<T>> levels;
   std::vector<void*> owned;
   // the solve as a list of steps, one launch each

@@ -236,8 +236,9 @@ stg_status stg_get_local_inverse(const stg_ctx* ctx, int level, long long cell, 
  * stream around the launches of the smoother's colour kernel on the finest
  * level (y_K = J_K^{-1} R_K r for the cells of one colour, Eq. (3.4)) in one
  * sweep per V-cycle (the last post-smoothing sweep, or the last pre-smoothing
- * sweep when nu2 = 0; the last sweep of stg_smooth) and accumulates their
- * device time; stg_profile(ctx, 0) stops and resets.  The
+ * sweep when nu2 = 0; the last sweep of stg_smooth), which is launched colour
+ * by colour for that (other sweeps take all patches in one launch), and
+ * accumulates their device time; stg_profile(ctx, 0) stops and resets.  The
  * V-cycle graph is recaptured when the setting changes.  stg_profile_read
  * returns the accumulated milliseconds, the number of launches and the number
  * of patches they processed (host pointers, each may be NULL). */
@@ -271,10 +272,10 @@ long long stg_kernel_launches(void);
  * STG_ECUDA on failure. */
 stg_status stg_invert_local_noalloc(int n, long long count, const double* a, double* a_inv, void* stream);
 
-/* Autotuner: times every variant of the smoother's colour kernel (one warp per
+/* Autotuner: times every variant of the smoother's patch kernel (one warp per
  * patch: 3 column-batch depths x 3 CTA sizes; factors staged in shared memory by
- * bulk copies: 4 pipeline shapes) on every level >= 1 and keeps the fastest per level; the
- * V-cycle graph is recaptured.  variant (host, may be NULL) receives the finest
+ * bulk copies: 4 pipeline shapes) on every level >= 1 and keeps the fastest per level (a
+ * later variant has to win by 2%); the V-cycle graph is recaptured.  variant (host, may be NULL) receives the finest
  * level's choice, sweep_ms (host, may be NULL) the finest level's time of one
  * sweep's colour kernels.  (Engineering service; the paper has no counterpart.) */
 stg_status stg_autotune(stg_ctx* ctx, int* variant, double* sweep_ms);

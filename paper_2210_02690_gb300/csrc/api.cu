@@ -196,7 +196,8 @@ struct LevelBufs {
   double* w = nullptr;
   double* asm_tab = nullptr;
   int colour_variant = kColourDefault;
-  void *b = nullptr, *x = nullptr, *r = nullptr, *z = nullptr;
+  void *b = nullptr, *x = nullptr, *r = nullptr;
+  void* y = nullptr;  // patch values of a sweep: n_cells x npatch (levels >= 1)
 };
 
 struct stg_ctx {
@@ -427,6 +428,8 @@ void apply64(stg_ctx* c, const LevelBufs& L, const double* x, const double* b, d
   apply_operator<double, double>(L.g, L.rowptr, L.colidx, L.vv, L.vp, L.pv, x, b, y, c->st);
 }
 
+// x_zero: the sweeps start from x = 0; x need not hold it (the first update writes every value), except
+// in the coloured mode, which adds into x.
 template <typename VT, typename FT>
 void smooth_level(stg_ctx* c, int l, int sweeps, bool x_zero) {
   LevelBufs& L = c->lv[l];
@@ -434,7 +437,7 @@ void smooth_level(stg_ctx* c, int l, int sweeps, bool x_zero) {
   VT* b = (VT*)L.b;
   VT* x = (VT*)L.x;
   VT* r = (VT*)L.r;
-  VT* z = (VT*)L.z;
+  VT* y = (VT*)L.y;
   const FT* jinv = (const FT*)L.jinv;
   const int ncol = 1 << g.dim;
   for (int s = 0; s < sweeps; ++s) {
@@ -449,18 +452,23 @@ void smooth_level(stg_ctx* c, int l, int sweeps, bool x_zero) {
         residual<VT>(c, L, x, b, r);
         res = r;
       }
-      for (int col = 0; col < ncol; ++col) {
-        const bool prof = prof_sweep && c->prof_on && l == (int)c->lv.size() - 1 &&
-                          c->prof_used + 2 <= (int)c->prof_ev.size();
-        if (prof) record_event(c->prof_ev[c->prof_used], c->st);
-        vanka_colour<VT, FT>(g, col, jinv, res, z, (VT)1, c->st, L.colour_variant);
-        if (prof) {
-          record_event(c->prof_ev[c->prof_used + 1], c->st);
-          c->prof_used += 2;
-          c->prof_pending_patches += g.coff[col + 1] - g.coff[col];
+      // one launch over all patches; a profiled sweep takes them colour by colour
+      if (prof_sweep && c->prof_on && l == (int)c->lv.size() - 1) {
+        for (int col = 0; col < ncol; ++col) {
+          const long long p0 = g.coff[col], cnt = g.coff[col + 1] - p0;
+          const bool prof = c->prof_used + 2 <= (int)c->prof_ev.size();
+          if (prof) record_event(c->prof_ev[c->prof_used], c->st);
+          vanka_patches<VT, FT>(g, p0, cnt, jinv, res, y, c->st, L.colour_variant);
+          if (prof) {
+            record_event(c->prof_ev[c->prof_used + 1], c->st);
+            c->prof_used += 2;
+            c->prof_pending_patches += cnt;
+          }
         }
+      } else {
+        vanka_patches<VT, FT>(g, 0, g.n_cells, jinv, res, y, c->st, L.colour_variant);
       }
-      vanka_update<VT>(g, x, z, c->opt.omega, c->st);
+      vanka_update<VT>(g, x, y, c->opt.omega, x_zero && s == 0, c->st);
     } else {
       for (int col = 0; col < ncol; ++col) {
         const VT* res = b;
@@ -530,7 +538,7 @@ void vcycle_level(stg_ctx* c, int l) {
   }
   LevelBufs& L = c->lv[l];
   LevelBufs& Lc = c->lv[l - 1];
-  fill_zero<VT>(L.g.N, (VT*)L.x, c->st);
+  if (c->opt.nu1 == 0 || c->opt.smoother == STG_VANKA_COLOURED) fill_zero<VT>(L.g.N, (VT*)L.x, c->st);
   smooth_level<VT, FT>(c, l, c->opt.nu1, true);
   residual<VT>(c, L, (const VT*)L.x, (const VT*)L.b, (VT*)L.r);
   restrict_res<VT>(Lc.g, L.g, (const VT*)L.r, (VT*)Lc.b, c->st);
@@ -822,19 +830,24 @@ double tune_level(stg_ctx* c, int l, int reps) {
   STG_CUDA_OK(cudaEventCreate(&e1));
   double best = 1e30;
   int bestv = L.colour_variant;
+  // a sweep's patches as the smoother launches them: all at once, or colour by colour (coloured mode)
+  const int parts = c->opt.smoother == STG_VANKA_AVERAGED ? 1 : 1 << L.g.dim;
+  auto sweep = [&](int v) {
+    for (int i = 0; i < parts; ++i) {
+      const long long p0 = parts == 1 ? 0 : L.g.coff[i], p1 = parts == 1 ? L.g.n_cells : L.g.coff[i + 1];
+      vanka_patches<VT, FT>(L.g, p0, p1 - p0, (const FT*)L.jinv, (const VT*)L.r, (VT*)L.y, c->st, v);
+    }
+  };
   for (int v = 0; v < kColourVariants; ++v) {
-    for (int w = 0; w < 2; ++w)  // warm-up
-      for (int col = 0; col < (1 << L.g.dim); ++col)
-        vanka_colour<VT, FT>(L.g, col, (const FT*)L.jinv, (const VT*)L.r, (VT*)L.z, (VT)1, c->st, v);
+    for (int w = 0; w < 2; ++w) sweep(v);  // warm-up
     STG_CUDA_OK(cudaEventRecord(e0, c->st));
-    for (int rep = 0; rep < reps; ++rep)
-      for (int col = 0; col < (1 << L.g.dim); ++col)
-        vanka_colour<VT, FT>(L.g, col, (const FT*)L.jinv, (const VT*)L.r, (VT*)L.z, (VT)1, c->st, v);
+    for (int rep = 0; rep < reps; ++rep) sweep(v);
     STG_CUDA_OK(cudaEventRecord(e1, c->st));
     STG_CUDA_OK(cudaEventSynchronize(e1));
     float ms = 0.f;
     STG_CUDA_OK(cudaEventElapsedTime(&ms, e0, e1));
-    if (ms / reps < best) {
+    // a later variant has to win by 2%: on small levels all are alike within the timer's noise
+    if (ms / reps < 0.98 * best) {
       best = ms / reps;
       bestv = v;
     }
@@ -842,7 +855,6 @@ double tune_level(stg_ctx* c, int l, int reps) {
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   L.colour_variant = bestv;
-  STG_CUDA_OK(cudaMemsetAsync(L.z, 0, (vc64(c) ? 8 : 4) * L.g.N, c->st));  // the smoother expects z = 0
   return best;
 }
 
@@ -991,10 +1003,9 @@ stg_status stg_setup(const stg_mesh* mesh, int k, double nu, double tau, const d
       L.b = dalloc<char>(c, (long long)vts * g.N);
       L.x = dalloc<char>(c, (long long)vts * g.N);
       L.r = dalloc<char>(c, (long long)vts * g.N);
-      L.z = dalloc<char>(c, (long long)vts * g.N);
-      STG_CUDA_OK(cudaMemset(L.z, 0, vts * g.N));
       STG_CUDA_OK(cudaMemset(L.x, 0, vts * g.N));
       if (l > 0) {
+        L.y = dalloc<char>(c, (long long)vts * g.n_cells * g.npatch);
         L.jinv = dalloc<char>(c, (long long)fsize(opt->factor_prec) * patch_stride(g.npatch) * g.n_cells);
         const int cf32 = opt->factor_prec != STG_F64 ? 1 : 0;
         if (l == mesh->n_levels - 1)

@@ -76,8 +76,8 @@ template <typename FT>
 bool invert_panels(const Geom& g, const int* rowptr, const double* vv, const double* vp, const double* pv, FT* jinv,
                    long long stride, int* flags, cudaStream_t st);
 
-// One colour phase of the smoother: y_K = J_K^{-1} R_K r for all cells of colour
-// `colour`; accumulate (averaged mode: z += y) or apply (coloured mode: z += omega y).
+// y_K = J_K^{-1} R_K r of the patches p0 .. p0 + cnt - 1, written to y[p npatch + row] (vanka_patches), or of one
+// colour, added into d with a factor (vanka_colour, the coloured mode).
 // variant = 3 * column-batch index (4, 8, 16 columns in flight) + CTA-size index (128, 256, 512)
 // Variants 0..8: one warp per patch, loads straight from global memory (3 column-batch depths x
 // 3 CTA sizes); 9..12: factors staged in shared memory by bulk copies (4 pipeline shapes), one
@@ -88,8 +88,11 @@ constexpr int kColourVariants = 17;
 constexpr int kColourWarpDefault = 4;  // 8 columns, 256 threads
 constexpr int kColourDefault = 9;      // 4 stages, 8 CTAs per SM (falls back to the warp form)
 template <typename VT, typename FT>
-void vanka_colour(const Geom& g, int colour, const FT* jinv, const VT* r, VT* z, VT scale, cudaStream_t st,
-                  int variant = kColourDefault);
+void vanka_patches(const Geom& g, long long p0, long long cnt, const FT* jinv, const VT* r, VT* y, cudaStream_t st,
+                   int variant);
+template <typename VT, typename FT>
+void vanka_colour(const Geom& g, int colour, const FT* jinv, const VT* r, VT* d, VT scale, cudaStream_t st,
+                  int variant);
 
 // Kronecker-split FP32 velocity rows (2D, 2..5 Radau nodes): per BCSR slot M_ij and the d x d
 // spatial blocks of every Radau node, split from the FP64 dense blocks.
@@ -105,9 +108,10 @@ bool colour_kernel_timed_out(cudaStream_t st);
 // Iteration limit of the staged colour kernel's waits for a factor copy.
 void set_colour_wait_limit(long long spins);
 
-// d += omega z / p (p = static multiplicity of (S2)); z = 0.
+// d += omega z / p (p = static multiplicity of (S2)), or d = omega z / p (from_zero), with z the sum of the patch
+// values y of vanka_patches at each DoF.
 template <typename VT>
-void vanka_update(const Geom& g, VT* d, VT* z, double omega, cudaStream_t st);
+void vanka_update(const Geom& g, VT* d, const VT* y, double omega, bool from_zero, cudaStream_t st);
 
 template <typename VT>
 void prolongate_add(const Geom& gc, const Geom& gf, const VT* xc, VT* xf, cudaStream_t st);

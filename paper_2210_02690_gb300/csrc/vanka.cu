@@ -3,12 +3,15 @@
 // Eq. (3.4): S_K(d) = R_K d + omega J_K^{-1} R_K (b - J d), with J_K the
 // restriction of the assembled J to the (k+1)(R^+S^) DoFs of cell K.  The
 // averaging loop (S0)-(S3) equals d <- d + omega (sum_K E_K J_K^{-1} R_K r) / p
-// with r = b - J d and p the number of cells sharing a DoF.  The sum is
-// accumulated colour by colour: cells of one colour share no velocity DoF and
-// pressure DoFs belong to one cell, so one colour's scatters never collide
-// (no atomics, deterministic order).
+// with r = b - J d and p the number of cells sharing a DoF.  The patches of a
+// sweep are independent given r: one launch writes every y_K = J_K^{-1} R_K r to
+// an array of its own (patch by patch), and the update sums each DoF's patches in
+// colour order (no atomics, deterministic).  The coloured (successive) mode adds
+// y_K into d colour by colour: cells of one colour share no velocity DoF and
+// pressure DoFs belong to one cell, so one colour's scatters never collide.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.cuh"
@@ -774,32 +777,61 @@ __global__ void __launch_bounds__(32 * WPB) __maxnreg__(MAXR)
 }
 
 // ------------------------------------------------------------------ smoother
-template <typename VT, typename FT, int RPL, int CB>
-__global__ void __launch_bounds__(512) vanka_colour_kernel(Geom g, int colour, const FT* __restrict__ jinv,
-                                                           long long stride, const VT* __restrict__ r,
-                                                           VT* __restrict__ z, VT scale) {
+// Local entry `row` of a patch: its offset from the patch's first velocity value (velocity rows) or
+// first pressure value, the same for every patch of a level.
+struct PatchRow {
+  int off;
+  bool vel;
+};
+__device__ __forceinline__ PatchRow patch_row(const Geom& g, int row) {
+  const int vel = g.nloc * g.NV;
+  if (row >= vel) return PatchRow{row - vel, false};
+  const int i = row / g.NV, v = row - i * g.NV, r1 = g.r + 1;
+  return PatchRow{((i % r1) + g.nn[0] * ((i / r1) % r1 + g.nn[1] * (i / (r1 * r1)))) * g.NV + v, true};
+}
+// First velocity and pressure value of patch p.  col: the colour of p or an earlier one, moved up to p's
+// (patches are ordered by colour).
+__device__ __forceinline__ void patch_bases(const Geom& g, long long p, int& col, long long& vb, long long& pb) {
+  while (p >= g.coff[col + 1]) ++col;
+  const unsigned li = (unsigned)(p - g.coff[col]), c0 = (unsigned)g.ccount[col][0], t = li / c0;
+  const int cx = 2 * (int)(li - t * c0) + (col & 1);
+  int cy, cz = 0;
+  if (g.dim == 2) {
+    cy = 2 * (int)t + (col >> 1);
+  } else {
+    const unsigned c1 = (unsigned)g.ccount[col][1], u = t / c1;
+    cy = 2 * (int)(t - u * c1) + ((col >> 1) & 1);
+    cz = 2 * (int)u + (col >> 2);
+  }
+  vb = node_id(g, g.r * cx, g.r * cy, g.r * cz) * g.NV;
+  pb = g.nvel + cell_id(g, cx, cy, cz) * g.NP;
+}
+
+// y_K = J_K^{-1} R_K r for the patches p0 .. p0 + cnt - 1, one warp per patch, loads straight from global
+// memory.  STORE: out[p n + row] = y (out: one block of n values per patch); otherwise out[dof] += scale y
+// (the patches of the range share no DoF).
+template <typename VT, typename FT, int RPL, int CB, bool STORE>
+__global__ void __launch_bounds__(512) vanka_colour_kernel(Geom g, long long p0, long long cnt,
+                                                           const FT* __restrict__ jinv, long long stride,
+                                                           const VT* __restrict__ r, VT* __restrict__ out, VT scale) {
   pdl_wait();
   using AT = typename AccT<VT>::type;
   const int n = g.npatch;
   const int wpb = blockDim.x >> 5, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long li = (long long)blockIdx.x * wpb + wid;
-  const long long cnt = g.coff[colour + 1] - g.coff[colour];
   extern __shared__ unsigned char smem_raw[];
   VT* rl = reinterpret_cast<VT*>(smem_raw) + wid * n;
   if (li >= cnt) return;
-  const long long p = g.coff[colour] + li;
-  const int* cc = g.ccount[colour];
-  long long rem = li;
-  const int jx = (int)(rem % cc[0]);
-  rem /= cc[0];
-  const int jy = (int)(rem % cc[1]);
-  const int jz = (int)(rem / cc[1]);
-  const int cx = 2 * jx + (colour & 1), cy = 2 * jy + ((colour >> 1) & 1), cz = 2 * jz + ((colour >> 2) & 1);
+  const long long p = p0 + li;
+  int col0 = 0;
+  long long vb, pb;
+  patch_bases(g, p, col0, vb, pb);
   long long gi[RPL];
 #pragma unroll
   for (int t = 0; t < RPL; ++t) {
     const int row = lane + 32 * t;
-    gi[t] = row < n ? patch_dof(g, cx, cy, cz, row) : 0;
+    const PatchRow pr = patch_row(g, row);
+    gi[t] = (pr.vel ? vb : pb) + pr.off;
     if (row < n) rl[row] = r[gi[t]];
   }
   __syncwarp();
@@ -837,12 +869,16 @@ __global__ void __launch_bounds__(512) vanka_colour_kernel(Geom g, int colour, c
 #pragma unroll
   for (int t = 0; t < RPL; ++t) {
     const int row = lane + 32 * t;
-    if (row < n) z[gi[t]] += scale * (VT)acc[t];
+    if (row >= n) continue;
+    if (STORE)
+      out[p * n + row] = (VT)acc[t];
+    else
+      out[gi[t]] += scale * (VT)acc[t];
   }
 }
 
 // ------------------------------------------------------------------ bulk-copy colour kernel
-// The same y_K = J_K^{-1} R_K r, z += y_K as vanka_colour_kernel, with each patch's factor
+// The same y_K = J_K^{-1} R_K r as vanka_colour_kernel, with each patch's factor
 // streamed into shared memory by the bulk-copy engine: one elected thread keeps S patches
 // in flight per CTA (cp.async.bulk completing on an mbarrier per stage) while the CTA, one
 // thread per row, computes the previous patch from shared memory.  Every wait has an
@@ -939,35 +975,28 @@ __device__ __forceinline__ void load_rows(const FT* p, AT (&a)[RPT]) {
   }
 }
 
-template <typename VT, typename FT, int S, int RPT>
-__global__ void __launch_bounds__(1024) vanka_colour_bulk_kernel(Geom g, int colour, const FT* __restrict__ jinv,
-                                                                 long long stride, const VT* __restrict__ r,
-                                                                 VT* __restrict__ z, VT scale, unsigned bytes,
-                                                                 unsigned stage_bytes) {
+template <typename VT, typename FT, int S, int RPT, bool STORE>
+__global__ void __launch_bounds__(1024) vanka_colour_bulk_kernel(Geom g, long long p0, long long cnt,
+                                                                 const FT* __restrict__ jinv, long long stride,
+                                                                 const VT* __restrict__ r, VT* __restrict__ out,
+                                                                 VT scale, unsigned bytes, unsigned stage_bytes) {
   pdl_wait();
   using AT = typename AccT<VT>::type;
-  extern __shared__ __align__(128) unsigned char smem_raw[];
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   const int n = g.npatch;
   const int tid = threadIdx.x;
-  const long long cnt = g.coff[colour + 1] - g.coff[colour];
   unsigned long long* bar = reinterpret_cast<unsigned long long*>(smem_raw);
   VT* rl = reinterpret_cast<VT*>(smem_raw + 128);  // two buffers of n values
   unsigned char* stages = smem_raw + 128 + bulk_rl_bytes<VT>(2 * n);
   const long long first = blockIdx.x, step = gridDim.x;
-  const FT* base = jinv + g.coff[colour] * stride;
-  const int* cc = g.ccount[colour];
+  const FT* base = jinv + p0 * stride;
   const long long spins = g_colour_wait_spins;
   // thread tid owns rows row0 .. row0 + RPT - 1 of every patch (RPT = 2 only for even n)
   const int row0 = tid * RPT;
   const bool act = row0 < n;
-  auto dof = [&](long long li, int row) {
-    long long rem = li;
-    const int jx = (int)(rem % cc[0]);
-    rem /= cc[0];
-    const int jy = (int)(rem % cc[1]);
-    const int jz = (int)(rem / cc[1]);
-    return patch_dof(g, 2 * jx + (colour & 1), 2 * jy + ((colour >> 1) & 1), 2 * jz + ((colour >> 2) & 1), row);
-  };
+  PatchRow pr[RPT];
+#pragma unroll
+  for (int u = 0; u < RPT; ++u) pr[u] = patch_row(g, act ? row0 + u : 0);
   if (tid == 0) {
     for (int s = 0; s < S; ++s) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar + s)));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -978,6 +1007,7 @@ __global__ void __launch_bounds__(1024) vanka_colour_bulk_kernel(Geom g, int col
     }
   }
   __syncthreads();  // no thread may poll a barrier before thread 0 has initialised it
+  int colour = 0;
   long long gi[RPT];
   VT zold[RPT];
 #pragma unroll
@@ -986,11 +1016,13 @@ __global__ void __launch_bounds__(1024) vanka_colour_bulk_kernel(Geom g, int col
     zold[u] = 0;
   }
   if (act && first < cnt) {
+    long long vb, pb;
+    patch_bases(g, p0 + first, colour, vb, pb);
 #pragma unroll
     for (int u = 0; u < RPT; ++u) {
-      gi[u] = dof(first, row0 + u);
+      gi[u] = (pr[u].vel ? vb : pb) + pr[u].off;
       rl[row0 + u] = r[gi[u]];
-      zold[u] = z[gi[u]];  // no other patch of this colour touches these entries
+      if (!STORE) zold[u] = out[gi[u]];  // no other patch of the range touches these entries
     }
   }
   int it = 0;
@@ -1026,11 +1058,13 @@ __global__ void __launch_bounds__(1024) vanka_colour_bulk_kernel(Geom g, int col
       zn[u] = 0;
     }
     if (act && ln < cnt) {
+      long long vb, pb;
+      patch_bases(g, p0 + ln, colour, vb, pb);
 #pragma unroll
       for (int u = 0; u < RPT; ++u) {
-        gn[u] = dof(ln, row0 + u);
+        gn[u] = (pr[u].vel ? vb : pb) + pr[u].off;
         rn[u] = r[gn[u]];
-        zn[u] = z[gn[u]];
+        if (!STORE) zn[u] = out[gn[u]];
       }
     }
     if (act) {
@@ -1049,7 +1083,10 @@ __global__ void __launch_bounds__(1024) vanka_colour_bulk_kernel(Geom g, int col
       }
 #pragma unroll
       for (int u = 0; u < RPT; ++u) {
-        z[gi[u]] = zold[u] + scale * (VT)acc[u];
+        if (STORE)
+          out[(p0 + li) * n + row0 + u] = (VT)acc[u];
+        else
+          out[gi[u]] = zold[u] + scale * (VT)acc[u];
         rl[((it + 1) & 1) * n + row0 + u] = rn[u];
       }
     }
@@ -1061,21 +1098,59 @@ __global__ void __launch_bounds__(1024) vanka_colour_bulk_kernel(Geom g, int col
   }
 }
 
+// d (+)= omega (sum of the DoF's patch values y) / p; the sum in colour order.  Bound by the latency of the
+// scattered reads of y (it was written just before and sits in L2).  With it a sweep is three launches (residual,
+// patches, update) where it was 2^d + 3, the patches run as one wave train instead of 2^d with a tail each, and the
+// read-modify-write of a z vector per patch becomes one store: 256^2 k = 3 step 48.9 -> 44.6 ms, 128 x 32 slab 7.5 -> 6.6 ms.
 template <typename VT>
-__global__ void vanka_update_kernel(Geom g, VT* __restrict__ d, VT* __restrict__ z, double omega) {
+__global__ void __launch_bounds__(256) vanka_update_kernel(Geom g, VT* __restrict__ d, const VT* __restrict__ y,
+                                                          double omega, int from_zero) {
   pdl_wait();
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= g.N) return;
+  const int n = g.npatch, r = g.r;
+  VT z;
   int mult = 1;
   if (t < g.nvel) {
-    const long long node = t / g.NV;
-    const int ix = (int)(node % g.nn[0]);
-    const int iy = (int)((node / g.nn[0]) % g.nn[1]);
-    const int iz = (int)(node / ((long long)g.nn[0] * g.nn[1]));
+    const unsigned NV = (unsigned)g.NV, node = t / NV, v = t - node * NV, nx = (unsigned)g.nn[0], w = node / nx;
+    const int ix = (int)(node - w * nx);
+    int iy = (int)w, iz = 0;
+    if (g.dim == 3) {
+      iz = (int)(w / (unsigned)g.nn[1]);
+      iy = (int)(w - (unsigned)iz * (unsigned)g.nn[1]);
+    }
     mult = node_multiplicity(g, ix, iy, iz);
+    int xl, xh, yl, yh, zl = 0, zh = 0;
+    node_cells(ix, g.n[0], xl, xh, r);
+    node_cells(iy, g.n[1], yl, yh, r);
+    if (g.dim == 3) node_cells(iz, g.n[2], zl, zh, r);
+    const int r1 = r + 1;
+    z = 0;
+    // even cells before odd ones along each direction: the colours in ascending order
+    for (int k = zl; k <= zh; ++k) {
+      const int cz = zl == zh ? zl : zl + (((k - zl) ^ (zl & 1)) & 1);
+      for (int j = yl; j <= yh; ++j) {
+        const int cy = yl == yh ? yl : yl + (((j - yl) ^ (yl & 1)) & 1);
+        for (int i = xl; i <= xh; ++i) {
+          const int cx = xl == xh ? xl : xl + (((i - xl) ^ (xl & 1)) & 1);
+          const int il = (ix - r * cx) + r1 * (iy - r * cy) + r1 * r1 * (iz - r * cz);
+          z += y[patch_of_cell(g, cx, cy, cz) * n + il * (int)NV + (int)v];
+        }
+      }
+    }
+  } else {
+    const unsigned u = t - (unsigned)g.nvel, NP = (unsigned)g.NP, cell = u / NP, q = u - cell * NP;
+    const unsigned nx = (unsigned)g.n[0], w = cell / nx;
+    const int cx = (int)(cell - w * nx);
+    int cy = (int)w, cz = 0;
+    if (g.dim == 3) {
+      cz = (int)(w / (unsigned)g.n[1]);
+      cy = (int)(w - (unsigned)cz * (unsigned)g.n[1]);
+    }
+    z = y[patch_of_cell(g, cx, cy, cz) * n + g.nloc * g.NV + (int)q];
   }
-  d[t] += (VT)omega * z[t] / (VT)mult;
-  z[t] = 0;
+  const VT dz = (VT)omega * z / (VT)mult;
+  d[t] = from_zero ? dz : d[t] + dz;
 }
 
 }  // namespace
@@ -1224,12 +1299,11 @@ struct BulkShape {
 constexpr BulkShape kBulkShapes[kColourVariants - kColourWarpVariants] = {
     {4, 32, 1}, {3, 32, 1}, {2, 32, 1}, {6, 32, 1}, {4, 32, 2}, {3, 32, 2}, {2, 32, 2}, {6, 32, 2}};
 
-template <typename VT, typename FT, int S, int RPT>
-bool launch_bulk(const Geom& g, int colour, const FT* jinv, const VT* r, VT* z, VT scale, cudaStream_t st,
-                 int ctas_per_sm) {
+template <typename VT, typename FT, int S, int RPT, bool STORE>
+bool launch_bulk(const Geom& g, long long p0, long long cnt, const FT* jinv, const VT* r, VT* out, VT scale,
+                 cudaStream_t st, int ctas_per_sm) {
   const int n = g.npatch;
   if (RPT == 2 && (n & 1)) return false;  // two rows per thread need an even patch size
-  const long long cnt = g.coff[colour + 1] - g.coff[colour];
   const long long stride = patch_stride(n);
   const unsigned bytes = (unsigned)((n * n * sizeof(FT) + 15) / 16 * 16);  // <= stride * sizeof(FT)
   const unsigned stage_bytes = (bytes + 127) / 128 * 128;
@@ -1242,11 +1316,11 @@ bool launch_bulk(const Geom& g, int colour, const FT* jinv, const VT* r, VT* z, 
   STG_CUDA_OK(cudaGetDevice(&dev));
   STG_CUDA_OK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   if (smem > 48 * 1024)
-    STG_CUDA_OK(cudaFuncSetAttribute(vanka_colour_bulk_kernel<VT, FT, S, RPT>,
+    STG_CUDA_OK(cudaFuncSetAttribute(vanka_colour_bulk_kernel<VT, FT, S, RPT, STORE>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
   // every CTA resident at once: the grid is capped by the occupancy the launch can reach
   int resident = 0;
-  STG_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, vanka_colour_bulk_kernel<VT, FT, S, RPT>,
+  STG_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, vanka_colour_bulk_kernel<VT, FT, S, RPT, STORE>,
                                                             threads, smem));
   if (resident < 1) return false;
   const long long want = (long long)sms * std::min(ctas_per_sm, resident);
@@ -1255,8 +1329,8 @@ bool launch_bulk(const Geom& g, int colour, const FT* jinv, const VT* r, VT* z, 
   // CTAs spread evenly over idle SMs; scheduled early into the SMs that the previous kernel frees
   // first, some SMs would take two CTAs and the launch would wait for them
   const OverlapScope serial(false);
-  launch_k(vanka_colour_bulk_kernel<VT, FT, S, RPT>, grid, threads, smem, st, g, colour, jinv, stride, r, z, scale, bytes,
-           stage_bytes);
+  launch_k(vanka_colour_bulk_kernel<VT, FT, S, RPT, STORE>, grid, threads, smem, st, g, p0, cnt, jinv, stride, r, out,
+           scale, bytes, stage_bytes);
   return true;
 }
 
@@ -1278,34 +1352,24 @@ bool colour_kernel_timed_out(cudaStream_t st) {
   return h != 0;
 }
 
-template <typename VT, typename FT>
-void vanka_colour(const Geom& g, int colour, const FT* jinv, const VT* r, VT* z, VT scale, cudaStream_t st,
-                  int variant) {
-  const long long cnt = g.coff[colour + 1] - g.coff[colour];
-  if (cnt == 0) return;
+namespace {
+
+template <typename VT, typename FT, bool STORE>
+void run_patches(const Geom& g, long long p0, long long cnt, const FT* jinv, const VT* r, VT* out, VT scale,
+                 cudaStream_t st, int variant) {
+  if (cnt <= 0) return;
   if (variant >= kColourWarpVariants) {
     const BulkShape b = kBulkShapes[(variant - kColourWarpVariants) % (kColourVariants - kColourWarpVariants)];
     bool done = false;
-    if (b.rows_per_thread == 2) {
-      if (b.stages == 2)
-        done = launch_bulk<VT, FT, 2, 2>(g, colour, jinv, r, z, scale, st, b.ctas_per_sm);
-      else if (b.stages == 3)
-        done = launch_bulk<VT, FT, 3, 2>(g, colour, jinv, r, z, scale, st, b.ctas_per_sm);
-      else if (b.stages == 4)
-        done = launch_bulk<VT, FT, 4, 2>(g, colour, jinv, r, z, scale, st, b.ctas_per_sm);
-      else
-        done = launch_bulk<VT, FT, 6, 2>(g, colour, jinv, r, z, scale, st, b.ctas_per_sm);
-    }
-    if (!done) {  // one row per thread (also for an odd patch size)
-      if (b.stages == 2)
-        done = launch_bulk<VT, FT, 2, 1>(g, colour, jinv, r, z, scale, st, b.ctas_per_sm);
-      else if (b.stages == 3)
-        done = launch_bulk<VT, FT, 3, 1>(g, colour, jinv, r, z, scale, st, b.ctas_per_sm);
-      else if (b.stages == 4)
-        done = launch_bulk<VT, FT, 4, 1>(g, colour, jinv, r, z, scale, st, b.ctas_per_sm);
-      else
-        done = launch_bulk<VT, FT, 6, 1>(g, colour, jinv, r, z, scale, st, b.ctas_per_sm);
-    }
+    auto staged = [&](auto rpt) {
+      constexpr int RPT = decltype(rpt)::value;
+      if (b.stages == 2) return launch_bulk<VT, FT, 2, RPT, STORE>(g, p0, cnt, jinv, r, out, scale, st, b.ctas_per_sm);
+      if (b.stages == 3) return launch_bulk<VT, FT, 3, RPT, STORE>(g, p0, cnt, jinv, r, out, scale, st, b.ctas_per_sm);
+      if (b.stages == 4) return launch_bulk<VT, FT, 4, RPT, STORE>(g, p0, cnt, jinv, r, out, scale, st, b.ctas_per_sm);
+      return launch_bulk<VT, FT, 6, RPT, STORE>(g, p0, cnt, jinv, r, out, scale, st, b.ctas_per_sm);
+    };
+    if (b.rows_per_thread == 2) done = staged(std::integral_constant<int, 2>{});
+    if (!done) done = staged(std::integral_constant<int, 1>{});  // also for an odd patch size
     if (done) return;
     variant = kColourWarpDefault;  // patch too large for the staged form
   }
@@ -1315,8 +1379,8 @@ void vanka_colour(const Geom& g, int colour, const FT* jinv, const VT* r, VT* z,
   const int threads = 128 << th_idx, wpb = threads / 32;
   const size_t sm = (size_t)wpb * n * sizeof(VT);
   const unsigned grid = grid_for(cnt, wpb);
-#define STG_VC(RPL, CB) \
-  launch_k(vanka_colour_kernel<VT, FT, RPL, CB>, grid, threads, sm, st, g, colour, jinv, stride, r, z, scale)
+#define STG_VC(RPL, CB)                                                                                             \
+  launch_k(vanka_colour_kernel<VT, FT, RPL, CB, STORE>, grid, threads, sm, st, g, p0, cnt, jinv, stride, r, out, scale)
 #define STG_VCB(RPL)      \
   if (cb_idx == 0)        \
     STG_VC(RPL, 4);       \
@@ -1341,9 +1405,23 @@ void vanka_colour(const Geom& g, int colour, const FT* jinv, const VT* r, VT* z,
 #undef STG_VC
 }
 
+}  // namespace
+
+template <typename VT, typename FT>
+void vanka_patches(const Geom& g, long long p0, long long cnt, const FT* jinv, const VT* r, VT* y, cudaStream_t st,
+                   int variant) {
+  run_patches<VT, FT, true>(g, p0, cnt, jinv, r, y, (VT)1, st, variant);
+}
+
+template <typename VT, typename FT>
+void vanka_colour(const Geom& g, int colour, const FT* jinv, const VT* r, VT* d, VT scale, cudaStream_t st,
+                  int variant) {
+  run_patches<VT, FT, false>(g, g.coff[colour], g.coff[colour + 1] - g.coff[colour], jinv, r, d, scale, st, variant);
+}
+
 template <typename VT>
-void vanka_update(const Geom& g, VT* d, VT* z, double omega, cudaStream_t st) {
-  launch_k(vanka_update_kernel<VT>, grid_for(g.N, 256), 256, 0, st, g, d, z, omega);
+void vanka_update(const Geom& g, VT* d, const VT* y, double omega, bool from_zero, cudaStream_t st) {
+  launch_k(vanka_update_kernel<VT>, grid_for(g.N, 256), 256, 0, st, g, d, y, omega, from_zero ? 1 : 0);
 }
 
 // explicit instantiations
@@ -1359,13 +1437,19 @@ template void invert_patches<float>(const Geom&, const int*, const double*, cons
 template void invert_patches<__nv_bfloat16>(const Geom&, const int*, const double*, const double*, const double*,
                                             const float*, const float*, const float*, __nv_bfloat16*, int, int*,
                                             void*, int*, cudaStream_t);
+template void vanka_patches<double, double>(const Geom&, long long, long long, const double*, const double*, double*,
+                                            cudaStream_t, int);
+template void vanka_patches<float, float>(const Geom&, long long, long long, const float*, const float*, float*,
+                                          cudaStream_t, int);
+template void vanka_patches<float, __nv_bfloat16>(const Geom&, long long, long long, const __nv_bfloat16*, const float*,
+                                                  float*, cudaStream_t, int);
 template void vanka_colour<double, double>(const Geom&, int, const double*, const double*, double*, double,
                                            cudaStream_t, int);
 template void vanka_colour<float, float>(const Geom&, int, const float*, const float*, float*, float, cudaStream_t,
                                          int);
 template void vanka_colour<float, __nv_bfloat16>(const Geom&, int, const __nv_bfloat16*, const float*, float*,
                                                  float, cudaStream_t, int);
-template void vanka_update<double>(const Geom&, double*, double*, double, cudaStream_t);
-template void vanka_update<float>(const Geom&, float*, float*, double, cudaStream_t);
+template void vanka_update<double>(const Geom&, double*, const double*, double, bool, cudaStream_t);
+template void vanka_update<float>(const Geom&, float*, const float*, double, bool, cudaStream_t);
 
 }  // namespace stg

@@ -217,7 +217,7 @@ struct stg_ctx {
   std::vector<LevelBufs> lv;
   CoarseSolver<double> coarse64;  // FP64 form
   CoarseSolver<float> coarse32;   // FP32 form: FP32 factors, FP64 iterative refinement
-  double *cb64 = nullptr, *cx64 = nullptr, *cr64 = nullptr, *cd64 = nullptr;
+  double *cb64 = nullptr, *cx64 = nullptr, *cr64 = nullptr;
   int* status = nullptr;
   void* inv_scratch = nullptr;
   int* inv_flags = nullptr;  // per patch: redo with pivoting
@@ -227,7 +227,7 @@ struct stg_ctx {
   float* mf_scr = nullptr;  // scratch of the matrix-free residual
   // FGMRES (finest level, internal layout, FP64)
   double *V = nullptr, *Z = nullptr, *wv = nullptr, *rv = nullptr, *partial = nullptr, *hd = nullptr;
-  double *vin = nullptr, *vout = nullptr, *tmp_a = nullptr, *tmp_b = nullptr;
+  double *tmp_a = nullptr, *tmp_b = nullptr;
   double* hh = nullptr;  // pinned host
   cudaGraphExec_t graph = nullptr;
   long long graph_kernels = 0;
@@ -496,7 +496,7 @@ void smooth_level(stg_ctx* c, int l, int sweeps, bool x_zero) {
 void coarse_solve64(stg_ctx* c, const double* b, double* x) {
   const LevelBufs& L = c->lv[0];
   if (coarse64(c)) {
-    c->coarse64.solve(b, x, c->st);
+    c->coarse64.solve(b, x, false, c->st);
     // The FP64 V-cycle refines its FP64 solve as well: the block cyclic reduction applies
     // explicit block inverses, whose forward error grows with cond(block) (observed relative
     // residuals around 5e-14 against about 1e-16 for an LU solve); each step with the FP64
@@ -505,35 +505,32 @@ void coarse_solve64(stg_ctx* c, const double* b, double* x) {
     if (vc64(c))
       for (int it = 0; it < c->opt.coarse_refine; ++it) {
         apply64(c, L, x, b, c->cr64);
-        c->coarse64.solve(c->cr64, c->cd64, c->st);
-        axpby(L.g.N, 1.0, c->cd64, 1.0, x, c->st);
+        c->coarse64.solve(c->cr64, x, true, c->st);
       }
     return;
   }
-  c->coarse32.solve(b, x, c->st);
+  c->coarse32.solve(b, x, false, c->st);
   for (int it = 0; it < c->opt.coarse_refine; ++it) {
     apply64(c, L, x, b, c->cr64);
-    c->coarse32.solve(c->cr64, c->cd64, c->st);
-    axpby(L.g.N, 1.0, c->cd64, 1.0, x, c->st);
+    c->coarse32.solve(c->cr64, x, true, c->st);
   }
 }
 
+// The coarsest level's vectors are FP64 in every form: b and x of the FP64 V-cycle's level 0, cb64 and cx64
+// under the FP32 V-cycle (the transfers widen and round).
 template <typename VT>
-void coarse_level(stg_ctx* c) {
-  LevelBufs& L = c->lv[0];
-  if (std::is_same<VT, double>::value) {
-    coarse_solve64(c, (const double*)L.b, (double*)L.x);
-  } else {
-    convert(L.g.N, (const float*)L.b, c->cb64, c->st);
-    coarse_solve64(c, c->cb64, c->cx64);
-    convert(L.g.N, c->cx64, (float*)L.x, c->st);
-  }
+double* coarse_b(stg_ctx* c) {
+  return std::is_same<VT, double>::value ? (double*)c->lv[0].b : c->cb64;
+}
+template <typename VT>
+double* coarse_x(stg_ctx* c) {
+  return std::is_same<VT, double>::value ? (double*)c->lv[0].x : c->cx64;
 }
 
 template <typename VT, typename FT>
 void vcycle_level(stg_ctx* c, int l) {
   if (l == 0) {
-    coarse_level<VT>(c);
+    coarse_solve64(c, coarse_b<VT>(c), coarse_x<VT>(c));
     return;
   }
   LevelBufs& L = c->lv[l];
@@ -541,29 +538,48 @@ void vcycle_level(stg_ctx* c, int l) {
   if (c->opt.nu1 == 0 || c->opt.smoother == STG_VANKA_COLOURED) fill_zero<VT>(L.g.N, (VT*)L.x, c->st);
   smooth_level<VT, FT>(c, l, c->opt.nu1, true);
   residual<VT>(c, L, (const VT*)L.x, (const VT*)L.b, (VT*)L.r);
-  restrict_res<VT>(Lc.g, L.g, (const VT*)L.r, (VT*)Lc.b, c->st);
+  if (l == 1)
+    restrict_res(Lc.g, L.g, (const VT*)L.r, coarse_b<VT>(c), c->st);
+  else
+    restrict_res(Lc.g, L.g, (const VT*)L.r, (VT*)Lc.b, c->st);
   vcycle_level<VT, FT>(c, l - 1);
-  prolongate_add<VT>(Lc.g, L.g, (const VT*)Lc.x, (VT*)L.x, c->st);
+  if (l == 1)
+    prolongate_add(Lc.g, L.g, (const double*)coarse_x<VT>(c), (VT*)L.x, c->st);
+  else
+    prolongate_add(Lc.g, L.g, (const VT*)Lc.x, (VT*)L.x, c->st);
   smooth_level<VT, FT>(c, l, c->opt.nu2, false);
 }
 
-// V-cycle from c->vin (FP64 internal) to c->vout (FP64 internal)
+// Input and output of the V-cycle on the finest level: its vectors b and x (FP64 internal layout outside).
+void vcycle_input(stg_ctx* c, const double* v) {
+  LevelBufs& F = c->lv.back();
+  if (c->lv.size() == 1 && !vc64(c))
+    STG_CUDA_OK(cudaMemcpyAsync(c->cb64, v, sizeof(double) * F.g.N, cudaMemcpyDeviceToDevice, c->st));
+  else if (vc64(c))
+    STG_CUDA_OK(cudaMemcpyAsync(F.b, v, sizeof(double) * F.g.N, cudaMemcpyDeviceToDevice, c->st));
+  else
+    convert(F.g.N, v, (float*)F.b, c->st);
+}
+void vcycle_output(stg_ctx* c, double* z) {
+  LevelBufs& F = c->lv.back();
+  if (c->lv.size() == 1 && !vc64(c))
+    STG_CUDA_OK(cudaMemcpyAsync(z, c->cx64, sizeof(double) * F.g.N, cudaMemcpyDeviceToDevice, c->st));
+  else if (vc64(c))
+    STG_CUDA_OK(cudaMemcpyAsync(z, F.x, sizeof(double) * F.g.N, cudaMemcpyDeviceToDevice, c->st));
+  else
+    convert(F.g.N, (const float*)F.x, z, c->st);
+}
+
+// V-cycle from the finest level's b to its x
 void vcycle_body(stg_ctx* c) {
   const OverlapScope overlap(c->opt.overlap_launches != 0);
-  LevelBufs& F = c->lv.back();
   const int top = (int)c->lv.size() - 1;
-  if (vc64(c)) {
-    STG_CUDA_OK(cudaMemcpyAsync(F.b, c->vin, sizeof(double) * F.g.N, cudaMemcpyDeviceToDevice, c->st));
+  if (vc64(c))
     vcycle_level<double, double>(c, top);
-    STG_CUDA_OK(cudaMemcpyAsync(c->vout, F.x, sizeof(double) * F.g.N, cudaMemcpyDeviceToDevice, c->st));
-  } else {
-    convert(F.g.N, c->vin, (float*)F.b, c->st);
-    if (c->opt.factor_prec == STG_F32)
-      vcycle_level<float, float>(c, top);
-    else
-      vcycle_level<float, __nv_bfloat16>(c, top);
-    convert(F.g.N, (const float*)F.x, c->vout, c->st);
-  }
+  else if (c->opt.factor_prec == STG_F32)
+    vcycle_level<float, float>(c, top);
+  else
+    vcycle_level<float, __nv_bfloat16>(c, top);
 }
 
 // One V-cycle; with profiling on, the events of the colour kernels are read
@@ -683,11 +699,7 @@ void fg_restart(FgState& S) {
 }
 
 // V-cycle input v_j
-void fg_pre(FgState& S) {
-  stg_ctx* c = S.c;
-  STG_CUDA_OK(cudaMemcpyAsync(c->vin, c->V + (long long)S.j * S.n, sizeof(double) * S.n, cudaMemcpyDeviceToDevice,
-                              c->st));
-}
+void fg_pre(FgState& S) { vcycle_input(S.c, S.c->V + (long long)S.j * S.n); }
 
 // z_j = V(v_j), w = J z_j, classical Gram-Schmidt twice, ||w||; the coefficients go to the host
 void fg_post(FgState& S) {
@@ -695,7 +707,7 @@ void fg_post(FgState& S) {
   const long long n = S.n;
   const int j = S.j;
   double* zj = c->Z + (long long)j * n;
-  STG_CUDA_OK(cudaMemcpyAsync(zj, c->vout, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->st));
+  vcycle_output(c, zj);
   apply_fine64(c, zj, c->wv);
   multi_dot(n, j + 1, c->V, n, c->wv, c->partial, c->hd, c->st);
   multi_axpy_sub(n, j + 1, c->V, n, c->hd, c->wv, c->st);
@@ -1026,7 +1038,6 @@ stg_status stg_setup(const stg_mesh* mesh, int k, double nu, double tau, const d
     c->cb64 = dalloc<double>(c, c->lv[0].g.N);
     c->cx64 = dalloc<double>(c, c->lv[0].g.N);
     c->cr64 = dalloc<double>(c, c->lv[0].g.N);
-    c->cd64 = dalloc<double>(c, c->lv[0].g.N);
     c->status = dalloc<int>(c, 4);
     const long long n = c->lv.back().g.N;
     const int m = opt->gmres_restart;
@@ -1034,8 +1045,6 @@ stg_status stg_setup(const stg_mesh* mesh, int k, double nu, double tau, const d
     c->Z = dalloc<double>(c, (long long)m * n);
     c->wv = dalloc<double>(c, n);
     c->rv = dalloc<double>(c, n);
-    c->vin = dalloc<double>(c, n);
-    c->vout = dalloc<double>(c, n);
     c->tmp_a = dalloc<double>(c, n);
     c->tmp_b = dalloc<double>(c, n);
     c->partial = dalloc<double>(c, (long long)dot_partial_doubles());
@@ -1134,9 +1143,11 @@ stg_status stg_vcycle(stg_ctx* c, const double* b, double* x) {
   if (!c || !b || !x) return STG_EINVAL;
   try {
     const Geom& g = c->lv.back().g;
-    cabi_to_internal<double>(g, b, c->vin, c->st);
+    cabi_to_internal<double>(g, b, c->tmp_a, c->st);
+    vcycle_input(c, c->tmp_a);
     run_vcycle(c);
-    internal_to_cabi<double>(g, c->vout, x, c->st);
+    vcycle_output(c, c->tmp_b);
+    internal_to_cabi<double>(g, c->tmp_b, x, c->st);
     if (c->prof_on) {
       STG_CUDA_OK(cudaStreamSynchronize(c->st));
       prof_collect(c);
@@ -1180,7 +1191,7 @@ stg_status stg_prolongate(stg_ctx* c, int level, const double* xc, double* xf) {
     const Geom& gf = c->lv[level].g;
     cabi_to_internal<double>(gc, xc, c->tmp_a, c->st);
     cabi_to_internal<double>(gf, xf, c->tmp_b, c->st);
-    prolongate_add<double>(gc, gf, c->tmp_a, c->tmp_b, c->st);
+    prolongate_add<double, double>(gc, gf, c->tmp_a, c->tmp_b, c->st);
     internal_to_cabi<double>(gf, c->tmp_b, xf, c->st);
     return STG_OK;
   } catch (const Error& e) {
@@ -1194,7 +1205,7 @@ stg_status stg_restrict(stg_ctx* c, int level, const double* rf, double* bc) {
     const Geom& gc = c->lv[level - 1].g;
     const Geom& gf = c->lv[level].g;
     cabi_to_internal<double>(gf, rf, c->tmp_a, c->st);
-    restrict_res<double>(gc, gf, c->tmp_a, c->tmp_b, c->st);
+    restrict_res<double, double>(gc, gf, c->tmp_a, c->tmp_b, c->st);
     internal_to_cabi<double>(gc, c->tmp_b, bc, c->st);
     return STG_OK;
   } catch (const Error& e) {

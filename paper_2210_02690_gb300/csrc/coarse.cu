@@ -381,12 +381,14 @@ __global__ void gather_rhs(CoarseView<T> v, const double* __restrict__ b, T* __r
 
 template <typename T>
 __global__ void scatter_sol(CoarseView<T> v, const T* __restrict__ xV, const T* __restrict__ xI,
-                            double* __restrict__ x) {
+                            double* __restrict__ x, int add) {
   pdl_wait();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= v.g.N) return;
   const Cls c = classify(v.g, v.mV, t);
-  x[t] = (double)(c.type == 0 ? xV[(long long)c.slab * v.mV + c.loc] : xI[(long long)c.slab * v.mI + c.loc]);
+  const double val =
+      (double)(c.type == 0 ? xV[(long long)c.slab * v.mV + c.loc] : xI[(long long)c.slab * v.mI + c.loc]);
+  x[t] = add ? x[t] + val : val;
 }
 
 template <typename T>
@@ -670,14 +672,14 @@ static void gemm2(int M, int N, int K, T alpha, const T* const* A0, const T* con
 
 // One plan step as a launch of its own.
 template <typename T>
-static void run_step(const CStep<T>& s, const CoarseView<T>& v, const double* b, double* x, T* bV, T* bI,
-                     const T* xV, const T* xI, cudaStream_t st) {
+static void run_step(const CStep<T>& s, const CoarseView<T>& v, const double* b, double* x, bool add, T* bV,
+                     T* bI, const T* xV, const T* xI, cudaStream_t st) {
   if (s.kind == kGather)
     launch_k(gather_rhs<T>, grid_for(v.g.N, 256), 256, 0, st, v, b, bV, bI);
   else if (s.kind == kMV)
     launch_k(bgemv2_kernel<T>, dim3((s.M + 7) / 8, s.batch), 256, 0, st, s);
   else
-    launch_k(scatter_sol<T>, grid_for(v.g.N, 256), 256, 0, st, v, xV, xI, x);
+    launch_k(scatter_sol<T>, grid_for(v.g.N, 256), 256, 0, st, v, xV, xI, x, add ? 1 : 0);
 }
 
 template <typename T>
@@ -728,8 +730,8 @@ void CoarseSolver<T>::factor(const int* rowptr, const int* colidx, const double*
 }
 
 template <typename T>
-void CoarseSolver<T>::solve(const double* b, double* x, cudaStream_t st) {
-  for (const CStep<T>& s : plan) run_step<T>(s, v, b, x, bV, bI, xV, xI, st);
+void CoarseSolver<T>::solve(const double* b, double* x, bool add, cudaStream_t st) {
+  for (const CStep<T>& s : plan) run_step<T>(s, v, b, x, add, bV, bI, xV, xI, st);
 }
 
 template <typename T>

@@ -55,7 +55,7 @@ struct CrLevel {
 //   kMV      y_i = alpha (A0_i x0_i + A1_i x1_i) + A2_i x2_i + c_i + beta y_i, i < batch, M rows
 //            per item (Ak: M x Nk row-major); a null array, or a null entry of one, drops its
 //            term
-//   kScatter xV, xI -> x (FP64, level layout)
+//   kScatter xV, xI -> x, or added into x (FP64, level layout)
 enum CoarseStepKind : int { kGather = 1, kMV = 2, kScatter = 4 };
 
 template <typename T>
@@ -92,8 +92,8 @@ struct CoarseSolver {
   // factor J_0 given in the internal level layout (FP64 operator), factors stored in T
   void factor(const int* rowptr, const int* colidx, const double* vv, const double* vp, const double* pv,
               cudaStream_t st);
-  // x = J_0^{-1} b, both FP64 in the internal level layout, arithmetic in T
-  void solve(const double* b, double* x, cudaStream_t st);
+  // x = J_0^{-1} b (add: x += J_0^{-1} b), both FP64 in the internal level layout, arithmetic in T
+  void solve(const double* b, double* x, bool add, cudaStream_t st);
   // 0 = ok, > 0: 1 + singular block, -1: coupling outside the block structure (synchronises)
   int read_status(cudaStream_t st);
 

@@ -113,10 +113,11 @@ void set_colour_wait_limit(long long spins);
 template <typename VT>
 void vanka_update(const Geom& g, VT* d, const VT* y, double omega, bool from_zero, cudaStream_t st);
 
-template <typename VT>
-void prolongate_add(const Geom& gc, const Geom& gf, const VT* xc, VT* xf, cudaStream_t st);
-template <typename VT>
-void restrict_res(const Geom& gc, const Geom& gf, const VT* rf, VT* bc, cudaStream_t st);
+// Transfers; the coarse vector's type may be FP64 under FP32 fine vectors (the coarsest level).
+template <typename XT, typename VT>
+void prolongate_add(const Geom& gc, const Geom& gf, const XT* xc, VT* xf, cudaStream_t st);
+template <typename VT, typename BT>
+void restrict_res(const Geom& gc, const Geom& gf, const VT* rf, BT* bc, cudaStream_t st);
 
 // C-ABI order <-> internal layout
 template <typename VT>

@@ -67,86 +67,76 @@ __device__ __forceinline__ int restrict_1d(int c, int nnf, int* idx, W* w) {
   return n;
 }
 
-template <typename VT>
-__global__ void prolong_vel(Geom gc, Geom gf, const VT* __restrict__ xc, VT* __restrict__ xf) {
+// xf += P xc: velocity and pressure of the fine level in one launch.  XT: the coarse vector's type (FP64 from
+// the coarsest level under the FP32 V-cycle, rounded as it is read).
+template <typename XT, typename VT>
+__global__ void prolong_kernel(Geom gc, Geom gf, const XT* __restrict__ xc, VT* __restrict__ xf) {
   pdl_wait();
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= gf.nvel) return;
-  const int NV = gf.NV;
-  const long long node = t / NV;
-  const int v = (int)(t - node * NV);
-  const int f[3] = {(int)(node % gf.nn[0]), (int)((node / gf.nn[0]) % gf.nn[1]),
-                    (int)(node / ((long long)gf.nn[0] * gf.nn[1]))};
-  if (gf.dim == 2 && node_dead(gf, f[0], f[1])) return;
-  int ix[3][3], n[3];
-  VT w[3][3];
-  for (int e = 0; e < 3; ++e) n[e] = prolong_1d<VT>(f[e], ix[e], w[e]);
-  VT acc = 0;
-  for (int c = 0; c < n[2]; ++c)
-    for (int b = 0; b < n[1]; ++b)
-      for (int a = 0; a < n[0]; ++a)
-        acc += w[0][a] * w[1][b] * w[2][c] * xc[node_id(gc, ix[0][a], ix[1][b], ix[2][c]) * NV + v];
-  xf[t] += acc;
-}
-
-template <typename VT>
-__global__ void prolong_pres(Geom gc, Geom gf, const VT* __restrict__ xc, VT* __restrict__ xf) {
-  pdl_wait();
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= gf.npres) return;
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= gf.N) return;
+  if (t < gf.nvel) {
+    const unsigned NV = (unsigned)gf.NV, node = t / NV, v = t - node * NV, nx = (unsigned)gf.nn[0], w_ = node / nx;
+    const unsigned ny = (unsigned)gf.nn[1], fz = gf.dim == 3 ? w_ / ny : 0u;
+    const int f[3] = {(int)(node - w_ * nx), (int)(w_ - fz * ny), (int)fz};
+    if (gf.dim == 2 && node_dead(gf, f[0], f[1])) return;
+    int ix[3][3], n[3];
+    VT w[3][3];
+    for (int e = 0; e < 3; ++e) n[e] = prolong_1d<VT>(f[e], ix[e], w[e]);
+    VT acc = 0;
+    for (int c = 0; c < n[2]; ++c)
+      for (int b = 0; b < n[1]; ++b)
+        for (int a = 0; a < n[0]; ++a)
+          acc += w[0][a] * w[1][b] * w[2][c] * (VT)xc[node_id(gc, ix[0][a], ix[1][b], ix[2][c]) * NV + v];
+    xf[t] += acc;
+    return;
+  }
   const int d = gf.dim;
-  const long long K = t / gf.NP;
-  const int q = (int)(t - K * gf.NP);
-  const int a = q / (d + 1), m = q % (d + 1);
-  const int f[3] = {(int)(K % gf.n[0]), (int)((K / gf.n[0]) % gf.n[1]), (int)(K / ((long long)gf.n[0] * gf.n[1]))};
+  const unsigned u = t - (unsigned)gf.nvel, NP = (unsigned)gf.NP, K = u / NP, q = u - K * NP;
+  const int a = (int)q / (d + 1), m = (int)q % (d + 1);
+  const unsigned nx = (unsigned)gf.n[0], w_ = K / nx, ny = (unsigned)gf.n[1], fz = d == 3 ? w_ / ny : 0u;
+  const int f[3] = {(int)(K - w_ * nx), (int)(w_ - fz * ny), (int)fz};
   if (d == 2 && cell_masked(gf, f[0], f[1])) return;
   const long long Kc = cell_id(gc, f[0] >> 1, f[1] >> 1, f[2] >> 1);
-  const VT* c = xc + gc.nvel + Kc * gc.NP + a * (d + 1);
+  const XT* c = xc + gc.nvel + Kc * gc.NP + a * (d + 1);
   VT val;
   if (m == 0) {
-    val = c[0];
-    for (int e = 0; e < d; ++e) val += ((f[e] & 1) ? (VT)0.5 : (VT)-0.5) * c[e + 1];
+    val = (VT)c[0];
+    for (int e = 0; e < d; ++e) val += ((f[e] & 1) ? (VT)0.5 : (VT)-0.5) * (VT)c[e + 1];
   } else {
-    val = (VT)0.5 * c[m];
+    val = (VT)0.5 * (VT)c[m];
   }
-  xf[gf.nvel + t] += val;
+  xf[t] += val;
 }
 
-template <typename VT>
-__global__ void restrict_vel(Geom gc, Geom gf, const VT* __restrict__ rf, VT* __restrict__ bc) {
+// bc = P^T rf, one launch; BT: the coarse vector's type (a widening of VT).
+template <typename VT, typename BT>
+__global__ void restrict_kernel(Geom gc, Geom gf, const VT* __restrict__ rf, BT* __restrict__ bc) {
   pdl_wait();
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= gc.nvel) return;
-  const int NV = gc.NV;
-  const long long node = t / NV;
-  const int v = (int)(t - node * NV);
-  const int c[3] = {(int)(node % gc.nn[0]), (int)((node / gc.nn[0]) % gc.nn[1]),
-                    (int)(node / ((long long)gc.nn[0] * gc.nn[1]))};
-  int ix[3][5], n[3];
-  VT w[3][5];
-  for (int e = 0; e < 3; ++e) n[e] = restrict_1d<VT>(c[e], gf.nn[e], ix[e], w[e]);
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= gc.N) return;
   VT acc = 0;
-  const bool obst = gf.dim == 2 && has_obstacle(gf);
-  for (int z = 0; z < n[2]; ++z)
-    for (int y = 0; y < n[1]; ++y)
-      for (int x = 0; x < n[0]; ++x) {
-        if (obst && node_dead(gf, ix[0][x], ix[1][y])) continue;
-        acc += w[0][x] * w[1][y] * w[2][z] * rf[node_id(gf, ix[0][x], ix[1][y], ix[2][z]) * NV + v];
-      }
-  bc[t] = acc;
-}
-
-template <typename VT>
-__global__ void restrict_pres(Geom gc, Geom gf, const VT* __restrict__ rf, VT* __restrict__ bc) {
-  pdl_wait();
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= gc.npres) return;
+  if (t < gc.nvel) {
+    const unsigned NV = (unsigned)gc.NV, node = t / NV, v = t - node * NV, nx = (unsigned)gc.nn[0], w_ = node / nx;
+    const unsigned ny = (unsigned)gc.nn[1], iz = gc.dim == 3 ? w_ / ny : 0u;
+    const int c[3] = {(int)(node - w_ * nx), (int)(w_ - iz * ny), (int)iz};
+    int ix[3][5], n[3];
+    VT w[3][5];
+    for (int e = 0; e < 3; ++e) n[e] = restrict_1d<VT>(c[e], gf.nn[e], ix[e], w[e]);
+    const bool obst = gf.dim == 2 && has_obstacle(gf);
+    for (int z = 0; z < n[2]; ++z)
+      for (int y = 0; y < n[1]; ++y)
+        for (int x = 0; x < n[0]; ++x) {
+          if (obst && node_dead(gf, ix[0][x], ix[1][y])) continue;
+          acc += w[0][x] * w[1][y] * w[2][z] * rf[node_id(gf, ix[0][x], ix[1][y], ix[2][z]) * NV + v];
+        }
+    bc[t] = (BT)acc;
+    return;
+  }
   const int d = gc.dim;
-  const long long K = t / gc.NP;
-  const int q = (int)(t - K * gc.NP);
-  const int a = q / (d + 1), m = q % (d + 1);
-  const int c[3] = {(int)(K % gc.n[0]), (int)((K / gc.n[0]) % gc.n[1]), (int)(K / ((long long)gc.n[0] * gc.n[1]))};
-  VT acc = 0;
+  const unsigned u = t - (unsigned)gc.nvel, NP = (unsigned)gc.NP, K = u / NP, q = u - K * NP;
+  const int a = (int)q / (d + 1), m = (int)q % (d + 1);
+  const unsigned nx = (unsigned)gc.n[0], w_ = K / nx, ny = (unsigned)gc.n[1], cz = d == 3 ? w_ / ny : 0u;
+  const int c[3] = {(int)(K - w_ * nx), (int)(w_ - cz * ny), (int)cz};
   const int nch = 1 << d;
   for (int o = 0; o < nch; ++o) {
     const int fx = 2 * c[0] + (o & 1), fy = d > 1 ? 2 * c[1] + ((o >> 1) & 1) : 0;
@@ -160,7 +150,7 @@ __global__ void restrict_pres(Geom gc, Geom gf, const VT* __restrict__ rf, VT* _
       acc += s * f[0] + (VT)0.5 * f[m];
     }
   }
-  bc[gc.nvel + t] = acc;
+  bc[t] = (BT)acc;
 }
 
 // ---------------------------------------------------------------- order 4 (2D)
@@ -211,74 +201,54 @@ __device__ __forceinline__ int restrict4_1d(int c, int nnf, int ncells, int* idx
   return n;
 }
 
-template <typename VT>
-__global__ void prolong_vel4(Geom gc, Geom gf, const VT* __restrict__ xc, VT* __restrict__ xf) {
+template <typename XT, typename VT>
+__global__ void prolong4_kernel(Geom gc, Geom gf, const XT* __restrict__ xc, VT* __restrict__ xf) {
   pdl_wait();
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= gf.nvel) return;
-  const int NV = gf.NV;
-  const long long node = t / NV;
-  const int v = (int)(t - node * NV);
-  const int fx = (int)(node % gf.nn[0]), fy = (int)(node / gf.nn[0]);
-  int ix[5], iy[5];
-  VT wx[5], wy[5];
-  const int nx = prolong4_1d<VT>(fx, ix, wx), ny = prolong4_1d<VT>(fy, iy, wy);
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= gf.N) return;
   VT acc = 0;
-  for (int b = 0; b < ny; ++b)
-    for (int a = 0; a < nx; ++a) acc += wx[a] * wy[b] * xc[node_id(gc, ix[a], iy[b], 0) * NV + v];
+  if (t < gf.nvel) {
+    const unsigned NV = (unsigned)gf.NV, node = t / NV, v = t - node * NV, nx_ = (unsigned)gf.nn[0], fy = node / nx_;
+    int ix[5], iy[5];
+    VT wx[5], wy[5];
+    const int nx = prolong4_1d<VT>((int)(node - fy * nx_), ix, wx), ny = prolong4_1d<VT>((int)fy, iy, wy);
+    for (int b = 0; b < ny; ++b)
+      for (int a = 0; a < nx; ++a) acc += wx[a] * wy[b] * (VT)xc[node_id(gc, ix[a], iy[b], 0) * NV + v];
+  } else {
+    const unsigned u = t - (unsigned)gf.nvel, NP = (unsigned)gf.NP, K = u / NP, q = u - K * NP;
+    const int a = (int)q / 10, m = (int)q % 10;
+    const unsigned nx_ = (unsigned)gf.n[0], fy = K / nx_, fx = K - fy * nx_;
+    const int o = (int)((fx & 1) + 2 * (fy & 1));
+    const XT* c = xc + gc.nvel + cell_id(gc, (int)(fx >> 1), (int)(fy >> 1), 0) * gc.NP + a * 10;
+    for (int j = 0; j < 10; ++j) acc += (VT)c_E4[o][m][j] * (VT)c[j];
+  }
   xf[t] += acc;
 }
 
-template <typename VT>
-__global__ void restrict_vel4(Geom gc, Geom gf, const VT* __restrict__ rf, VT* __restrict__ bc) {
+template <typename VT, typename BT>
+__global__ void restrict4_kernel(Geom gc, Geom gf, const VT* __restrict__ rf, BT* __restrict__ bc) {
   pdl_wait();
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= gc.nvel) return;
-  const int NV = gc.NV;
-  const long long node = t / NV;
-  const int v = (int)(t - node * NV);
-  const int cx = (int)(node % gc.nn[0]), cy = (int)(node / gc.nn[0]);
-  int ix[9], iy[9];
-  VT wx[9], wy[9];
-  const int nx = restrict4_1d<VT>(cx, gf.nn[0], gc.n[0], ix, wx);
-  const int ny = restrict4_1d<VT>(cy, gf.nn[1], gc.n[1], iy, wy);
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= gc.N) return;
   VT acc = 0;
-  for (int b = 0; b < ny; ++b)
-    for (int a = 0; a < nx; ++a) acc += wx[a] * wy[b] * rf[node_id(gf, ix[a], iy[b], 0) * NV + v];
-  bc[t] = acc;
-}
-
-template <typename VT>
-__global__ void prolong_pres4(Geom gc, Geom gf, const VT* __restrict__ xc, VT* __restrict__ xf) {
-  pdl_wait();
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= gf.npres) return;
-  const long long K = t / gf.NP;
-  const int q = (int)(t - K * gf.NP);
-  const int a = q / 10, m = q % 10;
-  const int fx = (int)(K % gf.n[0]), fy = (int)(K / gf.n[0]);
-  const int o = (fx & 1) + 2 * (fy & 1);
-  const VT* c = xc + gc.nvel + cell_id(gc, fx >> 1, fy >> 1, 0) * gc.NP + a * 10;
-  VT val = 0;
-  for (int j = 0; j < 10; ++j) val += (VT)c_E4[o][m][j] * c[j];
-  xf[gf.nvel + t] += val;
-}
-
-template <typename VT>
-__global__ void restrict_pres4(Geom gc, Geom gf, const VT* __restrict__ rf, VT* __restrict__ bc) {
-  pdl_wait();
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= gc.npres) return;
-  const long long K = t / gc.NP;
-  const int q = (int)(t - K * gc.NP);
-  const int a = q / 10, j = q % 10;
-  const int cx = (int)(K % gc.n[0]), cy = (int)(K / gc.n[0]);
-  VT acc = 0;
-  for (int o = 0; o < 4; ++o) {
-    const VT* f = rf + gf.nvel + cell_id(gf, 2 * cx + (o & 1), 2 * cy + (o >> 1), 0) * gf.NP + a * 10;
-    for (int m = 0; m < 10; ++m) acc += (VT)c_E4[o][m][j] * f[m];
+  if (t < gc.nvel) {
+    const unsigned NV = (unsigned)gc.NV, node = t / NV, v = t - node * NV, nx_ = (unsigned)gc.nn[0], cy = node / nx_;
+    int ix[9], iy[9];
+    VT wx[9], wy[9];
+    const int nx = restrict4_1d<VT>((int)(node - cy * nx_), gf.nn[0], gc.n[0], ix, wx);
+    const int ny = restrict4_1d<VT>((int)cy, gf.nn[1], gc.n[1], iy, wy);
+    for (int b = 0; b < ny; ++b)
+      for (int a = 0; a < nx; ++a) acc += wx[a] * wy[b] * rf[node_id(gf, ix[a], iy[b], 0) * NV + v];
+  } else {
+    const unsigned u = t - (unsigned)gc.nvel, NP = (unsigned)gc.NP, K = u / NP, q = u - K * NP;
+    const int a = (int)q / 10, j = (int)q % 10;
+    const unsigned nx_ = (unsigned)gc.n[0], cy = K / nx_, cx = K - cy * nx_;
+    for (int o = 0; o < 4; ++o) {
+      const VT* f = rf + gf.nvel + cell_id(gf, (int)(2 * cx) + (o & 1), (int)(2 * cy) + (o >> 1), 0) * gf.NP + a * 10;
+      for (int m = 0; m < 10; ++m) acc += (VT)c_E4[o][m][j] * f[m];
+    }
   }
-  bc[gc.nvel + t] = acc;
+  bc[t] = (BT)acc;
 }
 
 __device__ __forceinline__ long long cabi_index(const Geom& g, long long t) {
@@ -390,26 +360,20 @@ void upload_transfer4_tables() {
   STG_CUDA_OK(cudaMemcpyToSymbol(c_E4, E, sizeof(E)));
 }
 
-template <typename VT>
-void prolongate_add(const Geom& gc, const Geom& gf, const VT* xc, VT* xf, cudaStream_t st) {
-  if (gf.r == 4) {
-    launch_k(prolong_vel4<VT>, grid_for(gf.nvel, 256), 256, 0, st, gc, gf, xc, xf);
-    launch_k(prolong_pres4<VT>, grid_for(gf.npres, 256), 256, 0, st, gc, gf, xc, xf);
-    return;
-  }
-  launch_k(prolong_vel<VT>, grid_for(gf.nvel, 256), 256, 0, st, gc, gf, xc, xf);
-  launch_k(prolong_pres<VT>, grid_for(gf.npres, 256), 256, 0, st, gc, gf, xc, xf);
+template <typename XT, typename VT>
+void prolongate_add(const Geom& gc, const Geom& gf, const XT* xc, VT* xf, cudaStream_t st) {
+  if (gf.r == 4)
+    launch_k(prolong4_kernel<XT, VT>, grid_for(gf.N, 256), 256, 0, st, gc, gf, xc, xf);
+  else
+    launch_k(prolong_kernel<XT, VT>, grid_for(gf.N, 256), 256, 0, st, gc, gf, xc, xf);
 }
 
-template <typename VT>
-void restrict_res(const Geom& gc, const Geom& gf, const VT* rf, VT* bc, cudaStream_t st) {
-  if (gf.r == 4) {
-    launch_k(restrict_vel4<VT>, grid_for(gc.nvel, 256), 256, 0, st, gc, gf, rf, bc);
-    launch_k(restrict_pres4<VT>, grid_for(gc.npres, 256), 256, 0, st, gc, gf, rf, bc);
-    return;
-  }
-  launch_k(restrict_vel<VT>, grid_for(gc.nvel, 256), 256, 0, st, gc, gf, rf, bc);
-  launch_k(restrict_pres<VT>, grid_for(gc.npres, 256), 256, 0, st, gc, gf, rf, bc);
+template <typename VT, typename BT>
+void restrict_res(const Geom& gc, const Geom& gf, const VT* rf, BT* bc, cudaStream_t st) {
+  if (gf.r == 4)
+    launch_k(restrict4_kernel<VT, BT>, grid_for(gc.N, 256), 256, 0, st, gc, gf, rf, bc);
+  else
+    launch_k(restrict_kernel<VT, BT>, grid_for(gc.N, 256), 256, 0, st, gc, gf, rf, bc);
 }
 
 template <typename VT>
@@ -453,16 +417,17 @@ void convert(long long n, const S* in, D* out, cudaStream_t st) {
 
 template void fill_zero<double>(long long, double*, cudaStream_t);
 template void fill_zero<float>(long long, float*, cudaStream_t);
-template void prolongate_add<double>(const Geom&, const Geom&, const double*, double*, cudaStream_t);
-template void prolongate_add<float>(const Geom&, const Geom&, const float*, float*, cudaStream_t);
-template void restrict_res<double>(const Geom&, const Geom&, const double*, double*, cudaStream_t);
-template void restrict_res<float>(const Geom&, const Geom&, const float*, float*, cudaStream_t);
+template void prolongate_add<double, double>(const Geom&, const Geom&, const double*, double*, cudaStream_t);
+template void prolongate_add<float, float>(const Geom&, const Geom&, const float*, float*, cudaStream_t);
+template void prolongate_add<double, float>(const Geom&, const Geom&, const double*, float*, cudaStream_t);
+template void restrict_res<double, double>(const Geom&, const Geom&, const double*, double*, cudaStream_t);
+template void restrict_res<float, float>(const Geom&, const Geom&, const float*, float*, cudaStream_t);
+template void restrict_res<float, double>(const Geom&, const Geom&, const float*, double*, cudaStream_t);
 template void cabi_to_internal<double>(const Geom&, const double*, double*, cudaStream_t);
 template void cabi_to_internal<float>(const Geom&, const double*, float*, cudaStream_t);
 template void internal_to_cabi<double>(const Geom&, const double*, double*, cudaStream_t);
 template void internal_to_cabi<float>(const Geom&, const float*, double*, cudaStream_t);
 template void convert<float, double>(long long, const double*, float*, cudaStream_t);
 template void convert<double, float>(long long, const float*, double*, cudaStream_t);
-template void convert<__nv_bfloat16, double>(long long, const double*, __nv_bfloat16*, cudaStream_t);
 
 }  // namespace stg

@@ -25,14 +25,23 @@ template <>
 struct AccT<__nv_bfloat16> { using type = float; };
 
 // ------------------------------------------------------------------ J x, b - J x
+// Pressure row t of J x or b - J x.
 template <int DIM, typename MT, typename VT>
-__global__ void __launch_bounds__(256) op_vel_rows(Geom g, const int* __restrict__ rowptr,
-                                                   const int* __restrict__ colidx, const MT* __restrict__ vv,
-                                                   const MT* __restrict__ vp, const VT* __restrict__ x,
-                                                   const VT* __restrict__ b, VT* __restrict__ out) {
+__device__ __forceinline__ void op_pres_row(const Geom& g, const MT* __restrict__ pv, const VT* __restrict__ x,
+                                            const VT* __restrict__ b, VT* __restrict__ out, long long t);
+
+// Velocity rows (t < nvel) and pressure rows in one launch.
+template <int DIM, typename MT, typename VT>
+__global__ void __launch_bounds__(256) op_rows(Geom g, const int* __restrict__ rowptr, const int* __restrict__ colidx,
+                                               const MT* __restrict__ vv, const MT* __restrict__ vp,
+                                               const MT* __restrict__ pv, const VT* __restrict__ x,
+                                               const VT* __restrict__ b, VT* __restrict__ out) {
   pdl_wait();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= g.nvel) return;
+  if (t >= g.nvel) {
+    if (t < g.N) op_pres_row<DIM, MT, VT>(g, pv, x, b, out, t - g.nvel);
+    return;
+  }
   const int NV = g.NV;
   const long long node = t / NV;
   const int row = (int)(t - node * NV);
@@ -164,12 +173,16 @@ __device__ __forceinline__ void kron_stencil_row(const float* __restrict__ xj, c
 template <int NT>
 __global__ void __launch_bounds__(256) op_vel_rows_kron(Geom g, TimeF tf, const float* __restrict__ Mk,
                                                         const float* __restrict__ Ak,
-                                                        const float* __restrict__ vp, const float* __restrict__ x,
-                                                        const float* __restrict__ b, float* __restrict__ out) {
+                                                        const float* __restrict__ vp, const float* __restrict__ pv,
+                                                        const float* __restrict__ x, const float* __restrict__ b,
+                                                        float* __restrict__ out) {
   pdl_wait();
   constexpr int D = 2, NV = NT * D;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;  // (node, a) pairs < 2^31 (checked by the caller)
-  if (t >= g.n_nodes * NT) return;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;  // (node, a) pairs and pressure rows < 2^31 (caller)
+  if (t >= g.n_nodes * NT) {
+    if (t < g.n_nodes * NT + g.npres) op_pres_row<2, float, float>(g, pv, x, b, out, t - g.n_nodes * NT);
+    return;
+  }
   const int node = t / NT;
   const int a = t - node * NT;
   const int nx = g.nn[0];
@@ -230,11 +243,8 @@ __global__ void __launch_bounds__(256) op_vel_rows_kron(Geom g, TimeF tf, const 
 }
 
 template <int DIM, typename MT, typename VT>
-__global__ void __launch_bounds__(256) op_pres_rows(Geom g, const MT* __restrict__ pv, const VT* __restrict__ x,
-                                                    const VT* __restrict__ b, VT* __restrict__ out) {
-  pdl_wait();
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= g.npres) return;
+__device__ __forceinline__ void op_pres_row(const Geom& g, const MT* __restrict__ pv, const VT* __restrict__ x,
+                                            const VT* __restrict__ b, VT* __restrict__ out, long long t) {
   const long long K = t / g.NP;
   const int q = (int)(t - K * g.NP);
   const int npd = g.npd;
@@ -1158,13 +1168,11 @@ __global__ void __launch_bounds__(256) vanka_update_kernel(Geom g, VT* __restric
 template <typename MT, typename VT>
 void apply_operator(const Geom& g, const int* rowptr, const int* colidx, const MT* vv, const MT* vp, const MT* pv,
                     const VT* x, const VT* b, VT* out, cudaStream_t st) {
-  if (g.dim == 2) {
-    launch_k(op_vel_rows<2, MT, VT>, grid_for(g.nvel, 256), 256, 0, st, g, rowptr, colidx, vv, vp, x, b, out);
-    launch_k(op_pres_rows<2, MT, VT>, grid_for(g.npres, 256), 256, 0, st, g, pv, x, b, out);
-  } else {
-    launch_k(op_vel_rows<3, MT, VT>, grid_for(g.nvel, 256), 256, 0, st, g, rowptr, colidx, vv, vp, x, b, out);
-    launch_k(op_pres_rows<3, MT, VT>, grid_for(g.npres, 256), 256, 0, st, g, pv, x, b, out);
-  }
+  const unsigned grid = grid_for(g.N, 256);
+  if (g.dim == 2)
+    launch_k(op_rows<2, MT, VT>, grid, 256, 0, st, g, rowptr, colidx, vv, vp, pv, x, b, out);
+  else
+    launch_k(op_rows<3, MT, VT>, grid, 256, 0, st, g, rowptr, colidx, vv, vp, pv, x, b, out);
 }
 
 bool kron_supported(const Geom& g) { return g.dim == 2 && g.r == 2 && g.nt >= 2 && g.nt <= 5; }
@@ -1185,18 +1193,17 @@ void kron_split(const Geom& g, long long nnzb, const double* vv, const TimeData&
 void apply_operator_kron(const Geom& g, const TimeData& td, const float* Mk, const float* Ak,
                          const float* vp, const float* pv, const float* x, const float* b, float* out,
                          cudaStream_t st) {
-  if (g.n_nodes * g.nt >= (1LL << 31)) throw Error{STG_EINVAL, "level too large for 32-bit row indices"};
+  if (g.n_nodes * g.nt + g.npres >= (1LL << 31)) throw Error{STG_EINVAL, "level too large for 32-bit row indices"};
   TimeF tf;
   for (int a = 0; a < 5; ++a)
     for (int c = 0; c < 5; ++c) tf.T[a][c] = (float)td.T[a][c];
-  const unsigned grid = grid_for(g.n_nodes * g.nt, 256);
+  const unsigned grid = grid_for(g.n_nodes * g.nt + g.npres, 256);
   switch (g.nt) {
-    case 2: launch_k(op_vel_rows_kron<2>, grid, 256, 0, st, g, tf, Mk, Ak, vp, x, b, out); break;
-    case 3: launch_k(op_vel_rows_kron<3>, grid, 256, 0, st, g, tf, Mk, Ak, vp, x, b, out); break;
-    case 4: launch_k(op_vel_rows_kron<4>, grid, 256, 0, st, g, tf, Mk, Ak, vp, x, b, out); break;
-    default: launch_k(op_vel_rows_kron<5>, grid, 256, 0, st, g, tf, Mk, Ak, vp, x, b, out); break;
+    case 2: launch_k(op_vel_rows_kron<2>, grid, 256, 0, st, g, tf, Mk, Ak, vp, pv, x, b, out); break;
+    case 3: launch_k(op_vel_rows_kron<3>, grid, 256, 0, st, g, tf, Mk, Ak, vp, pv, x, b, out); break;
+    case 4: launch_k(op_vel_rows_kron<4>, grid, 256, 0, st, g, tf, Mk, Ak, vp, pv, x, b, out); break;
+    default: launch_k(op_vel_rows_kron<5>, grid, 256, 0, st, g, tf, Mk, Ak, vp, pv, x, b, out); break;
   }
-  launch_k(op_pres_rows<2, float, float>, grid_for(g.npres, 256), 256, 0, st, g, pv, x, b, out);
 }
 
 size_t invert_scratch_bytes(const Geom& g, int compute_f32) {

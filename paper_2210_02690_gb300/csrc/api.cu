@@ -190,6 +190,8 @@ struct LevelBufs {
   float *vv32 = nullptr, *vp32 = nullptr, *pv32 = nullptr;
   double* vconst = nullptr;  // the w = 0 assembly (time coupling, viscous, Nitsche), built once
   float *mk32 = nullptr, *ak32 = nullptr;  // Kronecker-split FP32 velocity rows (F32 form, levels >= 1, 2D)
+  void *op_lin = nullptr, *op_oseen = nullptr;  // coefficients of the matrix-free FP64 operator: the option's, Oseen's
+  const double* op_w = nullptr;  // velocity of the level's FP64 operator: w, or a Newton iterate's (then Oseen)
   float* w32 = nullptr;  // w and coefficients of the matrix-free FP32 residual (F32 form, levels >= 1, 3D and order 4)
   void* mf = nullptr;
   void* jinv = nullptr;
@@ -224,7 +226,8 @@ struct stg_ctx {
   // the same for the intermediate levels, which are inverted concurrently with the finest
   void* inv_scratch2 = nullptr;
   int* inv_flags2 = nullptr;
-  float* mf_scr = nullptr;  // scratch of the matrix-free residual
+  float* mf_scr = nullptr;     // scratch of the matrix-free residual
+  double* op_scr = nullptr;    // and of the matrix-free FP64 operator
   // FGMRES (finest level, internal layout, FP64)
   double *V = nullptr, *Z = nullptr, *wv = nullptr, *rv = nullptr, *partial = nullptr, *hd = nullptr;
   double *tmp_a = nullptr, *tmp_b = nullptr;
@@ -300,7 +303,7 @@ bool vc64(const stg_ctx* c) { return c->opt.vcycle_prec == STG_F64; }
 bool coarse64(const stg_ctx* c) { return vc64(c) || c->opt.coarse_prec == STG_F64; }
 
 // The part of every level's operator that does not depend on w, and the coefficients of the matrix-free
-// residual.
+// residual and operator.
 void assemble_constant(stg_ctx* c) {
   const AsmCoef cf0{c->nu, c->tau, c->opt.gamma1, c->opt.gamma2, 0};
   const AsmCoef cf{c->nu, c->tau, c->opt.gamma1, c->opt.gamma2, c->opt.linearisation == STG_NEWTON ? 1 : 0};
@@ -309,6 +312,8 @@ void assemble_constant(stg_ctx* c) {
     STG_CUDA_OK(cudaMemcpyAsync(L.vconst, L.vv, sizeof(double) * L.nnzb * L.g.NV * L.g.NV,
                                 cudaMemcpyDeviceToDevice, c->st));
     if (L.mf) residual_coef(L.g, c->td, cf, L.mf, c->st);
+    if (L.op_lin) operator_coef(L.g, c->td, cf, L.op_lin, c->st);
+    if (L.op_oseen) operator_coef(L.g, c->td, cf0, L.op_oseen, c->st);
   }
 }
 
@@ -316,6 +321,7 @@ void assemble_constant(stg_ctx* c) {
 // layout), invert the local matrices, factor the coarse system.
 void linearise_internal(stg_ctx* c) {
   const int nl = (int)c->lv.size();
+  for (LevelBufs& L : c->lv) L.op_w = L.w;
   for (int l = nl - 1; l > 0; --l) inject_w(c->lv[l - 1].g, c->lv[l].g, c->lv[l].w, c->lv[l - 1].w, c->st);
   AsmCoef cf{c->nu, c->tau, c->opt.gamma1, c->opt.gamma2, c->opt.linearisation == STG_NEWTON ? 1 : 0};
   STG_CUDA_OK(cudaMemsetAsync(c->status, 0, sizeof(int) * 4, c->st));
@@ -418,14 +424,19 @@ void residual(stg_ctx* c, const LevelBufs& L, const VT* x, const VT* b, VT* r) {
   else if (std::is_same<VT, float>::value && L.mk32)
     apply_operator_kron(L.g, c->td, L.mk32, L.ak32, L.vp32, L.pv32, (const float*)x, (const float*)b,
                         (float*)r, c->st);
+  else if (std::is_same<VT, double>::value && operator_mf_preferred(L.g))
+    operator_mf(L.g, L.op_lin, L.w, (const double*)x, (const double*)b, c->op_scr, (double*)r, c->st);
   else
     apply_operator<VT, VT>(L.g, L.rowptr, L.colidx, Ops<VT>::vv(L), Ops<VT>::vp(L), Ops<VT>::pv(L), x, b, r, c->st);
 }
 
-// J x (b null) or b - J x with the FP64 operator of level L.  The dense blocks stay: on GB300
-// the FP64 rows are bound by FP64 throughput, and the dense block needs the fewest operations.
+// J x (b null) or b - J x with the FP64 operator of level L: matrix-free in 3D (op_w: the level's w, or a Newton
+// iterate, whose Oseen operator is then never assembled), the assembled blocks otherwise and on the coarsest level.
 void apply64(stg_ctx* c, const LevelBufs& L, const double* x, const double* b, double* y) {
-  apply_operator<double, double>(L.g, L.rowptr, L.colidx, L.vv, L.vp, L.pv, x, b, y, c->st);
+  if (operator_mf_preferred(L.g) && (&L != &c->lv[0] || L.op_w != L.w))
+    operator_mf(L.g, L.op_w != L.w ? L.op_oseen : L.op_lin, L.op_w, x, b, c->op_scr, y, c->st);
+  else
+    apply_operator<double, double>(L.g, L.rowptr, L.colidx, L.vv, L.vp, L.pv, x, b, y, c->st);
 }
 
 // x_zero: the sweeps start from x = 0; x need not hold it (the first update writes every value), except
@@ -504,14 +515,14 @@ void coarse_solve64(stg_ctx* c, const double* b, double* x) {
     // are used as they are.
     if (vc64(c))
       for (int it = 0; it < c->opt.coarse_refine; ++it) {
-        apply64(c, L, x, b, c->cr64);
+        apply_operator<double, double>(L.g, L.rowptr, L.colidx, L.vv, L.vp, L.pv, x, b, c->cr64, c->st);
         c->coarse64.solve(c->cr64, x, true, c->st);
       }
     return;
   }
   c->coarse32.solve(b, x, false, c->st);
   for (int it = 0; it < c->opt.coarse_refine; ++it) {
-    apply64(c, L, x, b, c->cr64);
+    apply_operator<double, double>(L.g, L.rowptr, L.colidx, L.vv, L.vp, L.pv, x, b, c->cr64, c->st);
     c->coarse32.solve(c->cr64, x, true, c->st);
   }
 }
@@ -783,14 +794,18 @@ stg_status fgmres(stg_ctx* c, const double* b, double* x, int* iters_out, double
   return fg_result(S, iters_out, rel_out);
 }
 
-// r = b - F... precisely r = -F_n(X) = b - J_Oseen(w = v(X)) X on the finest level (the finest
-// operator storage is overwritten by the Oseen Jacobian at v(X)).
+// r = -F_n(X) = b - J_Oseen(w = v(X)) X on the finest level, whose FP64 operator that Oseen Jacobian becomes (until the
+// next linearisation).
 double neg_residual(stg_ctx* c, const double* X, double* r) {
   LevelBufs& F = c->lv.back();
-  AsmCoef cf{c->nu, c->tau, c->opt.gamma1, c->opt.gamma2, 0};
   // the velocity part of an internal vector is laid out exactly like an internal w
-  assemble_level_w(F.g, c->td, cf, X, F.rowptr, F.asm_tab, F.vconst, F.vv, F.nnzb, c->st);
-  apply_operator<double, double>(F.g, F.rowptr, F.colidx, F.vv, F.vp, F.pv, X, c->nb, r, c->st);
+  if (operator_mf_preferred(F.g)) {
+    F.op_w = X;
+  } else {
+    const AsmCoef cf{c->nu, c->tau, c->opt.gamma1, c->opt.gamma2, 0};
+    assemble_level_w(F.g, c->td, cf, X, F.rowptr, F.asm_tab, F.vconst, F.vv, F.nnzb, c->st);
+  }
+  apply64(c, F, X, c->nb, r);
   return std::sqrt(dot_host(c, r, r));
 }
 
@@ -1010,6 +1025,10 @@ stg_status stg_setup(const stg_mesh* mesh, int k, double nu, double tau, const d
         }
       }
       L.w = dalloc<double>(c, g.nvel);
+      if (operator_mf_preferred(g)) {
+        L.op_lin = dalloc<char>(c, (long long)residual_coef_bytes());
+        L.op_oseen = dalloc<char>(c, (long long)residual_coef_bytes());
+      }
       L.asm_tab = dalloc<double>(c, assemble_table_doubles(g.dim, k));
       L.vconst = dalloc<double>(c, L.nnzb * g.NV * g.NV);
       L.b = dalloc<char>(c, (long long)vts * g.N);
@@ -1028,6 +1047,7 @@ stg_status stg_setup(const stg_mesh* mesh, int k, double nu, double tau, const d
     }
     if (scratch) c->inv_scratch = dalloc<char>(c, (long long)scratch);
     if (scratch2) c->inv_scratch2 = dalloc<char>(c, (long long)scratch2);
+    if (c->lv.back().op_lin) c->op_scr = dalloc<double>(c, residual_scratch(c->lv.back().g));
     if (c->lv.back().mf) c->mf_scr = dalloc<float>(c, residual_scratch(c->lv.back().g));
     c->inv_flags = dalloc<int>(c, c->lv.back().g.n_cells);
     if (mesh->n_levels > 2) c->inv_flags2 = dalloc<int>(c, c->lv[mesh->n_levels - 2].g.n_cells);

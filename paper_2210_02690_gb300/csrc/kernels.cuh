@@ -60,6 +60,13 @@ void residual_coef(const Geom& g, const TimeData& td, const AsmCoef& cf, void* d
 void residual_mf(const Geom& g, const void* coef, const float* w, const float* x, const float* b, float* scratch,
                  float* out, cudaStream_t st);
 
+// The FP64 operator without a matrix (3D, residual64.cu): out = b - J x, or J x (b null), at linearisation velocity w (FP64,
+// internal layout); coef as above, scratch: residual_scratch(g) doubles.
+bool operator_mf_preferred(const Geom& g);
+void operator_coef(const Geom& g, const TimeData& td, const AsmCoef& cf, void* dst, cudaStream_t st);
+void operator_mf(const Geom& g, const void* coef, const double* w, const double* x, const double* b, double* scratch,
+                 double* out, cudaStream_t st);
+
 // Local inverses J_K^{-1} of every cell (gather from the assembled J, Gauss-Jordan
 // with partial pivoting in CT precision, stored as FT). status[0] receives the
 // first singular cell + 1 (0 = none).

@@ -197,7 +197,7 @@ struct LevelBufs {
   void* jinv = nullptr;
   double* w = nullptr;
   double* asm_tab = nullptr;
-  int colour_variant = kColourDefault;
+  int colour_variant = 0;
   void *b = nullptr, *x = nullptr, *r = nullptr;
   void* y = nullptr;  // patch values of a sweep: n_cells x npatch (levels >= 1)
 };
@@ -1036,6 +1036,7 @@ stg_status stg_setup(const stg_mesh* mesh, int k, double nu, double tau, const d
       L.r = dalloc<char>(c, (long long)vts * g.N);
       STG_CUDA_OK(cudaMemset(L.x, 0, vts * g.N));
       if (l > 0) {
+        L.colour_variant = default_colour_variant(g, opt->factor_prec);
         L.y = dalloc<char>(c, (long long)vts * g.n_cells * g.npatch);
         L.jinv = dalloc<char>(c, (long long)fsize(opt->factor_prec) * patch_stride(g.npatch) * g.n_cells);
         const int cf32 = opt->factor_prec != STG_F64 ? 1 : 0;

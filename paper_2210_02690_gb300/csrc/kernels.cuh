@@ -93,7 +93,8 @@ bool invert_panels(const Geom& g, const int* rowptr, const double* vv, const dou
 constexpr int kColourWarpVariants = 9;
 constexpr int kColourVariants = 17;
 constexpr int kColourWarpDefault = 4;  // 8 columns, 256 threads
-constexpr int kColourDefault = 9;      // 4 stages, 8 CTAs per SM (falls back to the warp form)
+// The variant a level starts with; the autotuner may replace it.
+int default_colour_variant(const Geom& g, int factor_prec);
 template <typename VT, typename FT>
 void vanka_patches(const Geom& g, long long p0, long long cnt, const FT* jinv, const VT* r, VT* y, cudaStream_t st,
                    int variant);

@@ -1414,6 +1414,18 @@ void run_patches(const Geom& g, long long p0, long long cnt, const FT* jinv, con
 
 }  // namespace
 
+// Two stages keep the most CTAs on an SM, and bytes in flight are what the staged form needs; the factor may be
+// large before one or two CTAs are left (44 KB at n = 105 in FP32).  Beyond, and in FP64 from n = 60 on (bound by the
+// FP64 pipe), one warp per patch.  Whole sweeps (residual and update included) on 65536 patches, 4 stages
+// -> this choice: FP32 n = 63 299 -> 280 us, 84 464 -> 450, 105 814 -> 652 (one warp per patch 687); BF16, whose
+// issue-bound product wants two rows a thread, n = 42 (90112) 202 -> 173, 84 387 -> 330, 105 572 -> 461; FP64 n = 63
+// 1886 -> 966.  3D n = 85, 32768 patches: FP32 349 -> 213.  FP32 n = 120, 170: two stages 301, 329, one warp 284, 323.
+int default_colour_variant(const Geom& g, int factor_prec) {
+  const int n = g.npatch, size = factor_prec == STG_F64 ? 8 : (factor_prec == STG_F32 ? 4 : 2);
+  if (factor_prec == STG_F64 ? n < 60 : n * n * size <= 48 * 1024) return factor_prec == STG_BF16 ? 15 : 11;
+  return 3;
+}
+
 template <typename VT, typename FT>
 void vanka_patches(const Geom& g, long long p0, long long cnt, const FT* jinv, const VT* r, VT* y, cudaStream_t st,
                    int variant) {

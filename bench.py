@@ -293,11 +293,11 @@ FP64_NOMINAL_TFLOPS = 1.25  # GB300 dense FP64, nominal
 def colour_fraction(k: int, form: str, ms: float, launches: int, patches: int, peak: float,
                     variant: int | None = None) -> dict:
     """HBM fraction of the finest level's colour kernels (2D): algorithmic bytes (every J_K^{-1}
-    in the form's factor precision, r gathered, z read and written) over their CUDA-event time."""
+    in the form's factor precision, r gathered, y stored) over their CUDA-event time."""
     n = 21 * (k + 1)
     fs = {"f64": 8, "f32": 4, "bf16": 2}[form]
     vs = 8 if form == "f64" else 4
-    per_launch = n * (n * fs + 3 * vs) * patches / max(launches, 1)
+    per_launch = n * (n * fs + 2 * vs) * patches / max(launches, 1)
     avg = ms / max(launches, 1)
     gbs = per_launch / (avg * 1e-3) / 1e9 if avg > 0 else 0.0
     out = {"bytes_per_launch": per_launch, "avg_launch_ms": avg, "gbs": gbs, "frac": gbs / peak,
@@ -466,8 +466,8 @@ def gpu_arm(args) -> None:
     pms, plaunch, ppatch = r32["colour_kernel"]
     npatch = 21 * (k + 1)
     # algorithmic bytes of one colour-kernel launch: each patch streams its J_K^{-1}
-    # (npatch^2 FP32 values), gathers npatch residual values and reads+writes npatch values of z
-    bytes_per_patch = npatch * npatch * 4 + 3 * npatch * 4
+    # (npatch^2 FP32 values), gathers npatch residual values and stores npatch values of y
+    bytes_per_patch = npatch * npatch * 4 + 2 * npatch * 4
     avg_ms = pms / max(plaunch, 1)
     per_launch_bytes = bytes_per_patch * ppatch / max(plaunch, 1)
     achieved = per_launch_bytes / (avg_ms * 1e-3) / 1e9 if avg_ms > 0 else 0.0

@@ -1169,10 +1169,13 @@ template <typename MT, typename VT>
 void apply_operator(const Geom& g, const int* rowptr, const int* colidx, const MT* vv, const MT* vp, const MT* pv,
                     const VT* x, const VT* b, VT* out, cudaStream_t st) {
   const unsigned grid = grid_for(g.N, 256);
-  if (g.dim == 2)
+  if (g.dim == 2) {
     launch_k(op_rows<2, MT, VT>, grid, 256, 0, st, g, rowptr, colidx, vv, vp, pv, x, b, out);
-  else
+  } else if constexpr (sizeof(MT) == 8) {
     launch_k(op_rows<3, MT, VT>, grid, 256, 0, st, g, rowptr, colidx, vv, vp, pv, x, b, out);
+  } else {
+    throw Error{STG_EINVAL, "FP32 3D levels apply their operator without a matrix"};
+  }
 }
 
 bool kron_supported(const Geom& g) { return g.dim == 2 && g.r == 2 && g.nt >= 2 && g.nt <= 5; }
@@ -1241,13 +1244,10 @@ void invert_patches(const Geom& g, const int* rowptr, const double* vv, const do
     // 2.  The 168 cap costs a few spill slots outside the elimination loop and measured faster
     // than both the spill-free 200 cap and the two-rows-per-thread CTA kernel this replaced
     // (finest channel set-up 4.98 ms against 5.23 and 5.29 ms).
-    if (vv32) {
-      if (n == 21) run(invert_triples_kernel<21, 4, 128, float, FT>, 16, 128, vv32, vp32, pv32);
-      else run(invert_triples_kernel<42, 2, 168, float, FT>, 4, 64, vv32, vp32, pv32);
-    } else {
-      if (n == 21) run(invert_triples_kernel<21, 4, 128, double, FT>, 16, 128, vv, vp, pv);
-      else run(invert_triples_kernel<42, 2, 168, double, FT>, 4, 64, vv, vp, pv);
-    }
+    // n = 21 (k = 0) is the one size without the Kronecker split, so it has the FP32 blocks at
+    // hand; n = 42 has only the FP64 blocks and rounds them as it gathers
+    if (n == 21) run(invert_triples_kernel<21, 4, 128, float, FT>, 16, 128, vv32, vp32, pv32);
+    else run(invert_triples_kernel<42, 2, 168, double, FT>, 4, 64, vv, vp, pv);
     only = flags;
   } else if (compute_f32 && flags && invert_panels<FT>(g, rowptr, vv, vp, pv, jinv, stride, flags, st)) {
     only = flags;  // blocked register elimination, pivot-free; the pivoting kernel redoes flagged patches

@@ -1183,24 +1183,23 @@ template <typename MT, typename VT>
 void apply_operator(const Geom& g, const int* rowptr, const int* colidx, const MT* vv, const MT* vp, const MT* pv,
                     const VT* x, const VT* b, VT* out, cudaStream_t st) {
   const unsigned grid = grid_for(g.N, 256);
-  auto run = [&](auto kern) { launch_k(kern, grid, 256, 0, st, g, rowptr, colidx, vv, vp, pv, x, b, out); };
   if constexpr (sizeof(MT) == 4) {
     // the other FP32 levels take the Kronecker split (2D) or no matrix (3D, order 4)
     if (g.dim != 2 || g.nt != 1) throw Error{STG_EINVAL, "no assembled FP32 operator on this level"};
-    run(op_rows<2, 1, MT, VT>);
+    launch_k(op_rows<2, 1, MT, VT>, grid, 256, 0, st, g, rowptr, colidx, vv, vp, pv, x, b, out);
   } else if (g.dim == 2) {
     switch (g.nt) {
-      case 1: run(op_rows<2, 1, MT, VT>); break;
-      case 2: run(op_rows<2, 2, MT, VT>); break;
-      case 3: run(op_rows<2, 3, MT, VT>); break;
-      case 4: run(op_rows<2, 4, MT, VT>); break;
-      default: run(op_rows<2, 5, MT, VT>); break;
+      case 1: launch_k(op_rows<2, 1, MT, VT>, grid, 256, 0, st, g, rowptr, colidx, vv, vp, pv, x, b, out); break;
+      case 2: launch_k(op_rows<2, 2, MT, VT>, grid, 256, 0, st, g, rowptr, colidx, vv, vp, pv, x, b, out); break;
+      case 3: launch_k(op_rows<2, 3, MT, VT>, grid, 256, 0, st, g, rowptr, colidx, vv, vp, pv, x, b, out); break;
+      case 4: launch_k(op_rows<2, 4, MT, VT>, grid, 256, 0, st, g, rowptr, colidx, vv, vp, pv, x, b, out); break;
+      default: launch_k(op_rows<2, 5, MT, VT>, grid, 256, 0, st, g, rowptr, colidx, vv, vp, pv, x, b, out); break;
     }
   } else {
     switch (g.nt) {
-      case 1: run(op_rows<3, 1, MT, VT>); break;
-      case 2: run(op_rows<3, 2, MT, VT>); break;
-      default: run(op_rows<3, 3, MT, VT>); break;
+      case 1: launch_k(op_rows<3, 1, MT, VT>, grid, 256, 0, st, g, rowptr, colidx, vv, vp, pv, x, b, out); break;
+      case 2: launch_k(op_rows<3, 2, MT, VT>, grid, 256, 0, st, g, rowptr, colidx, vv, vp, pv, x, b, out); break;
+      default: launch_k(op_rows<3, 3, MT, VT>, grid, 256, 0, st, g, rowptr, colidx, vv, vp, pv, x, b, out); break;
     }
   }
 }

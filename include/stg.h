@@ -167,6 +167,10 @@ stg_status stg_vcycle(stg_ctx* ctx, const double* b, double* x);
  * place ((S0)-(S3) for STG_VANKA_AVERAGED).  Runs in the V-cycle precision. */
 stg_status stg_smooth(stg_ctx* ctx, int level, int sweeps, const double* b, double* x);
 
+/* r = b - J_l x on level `level` >= 1 as the V-cycle computes it: with vcycle_prec STG_F32 in FP32, x and b
+ * rounded to it (engineering service: the rounding error of that residual). */
+stg_status stg_level_residual(stg_ctx* ctx, int level, const double* b, const double* x, double* r);
+
 /* Grid transfer (nested FE spaces; time nodes are not coarsened):
  * stg_prolongate: x_fine += P x_coarse; stg_restrict: b_coarse = P^T r_fine.
  * `level` is the FINE level (>= 1); vectors in the levels' C-ABI orders. */

@@ -27,7 +27,7 @@ PREC = {"f64": STG_F64, "f32": STG_F32, "bf16": STG_BF16}
 
 EXPORTED = ("stg_options_default", "stg_setup", "stg_update_linearisation", "stg_set_slab_length",
             "stg_apply_jacobian",
-            "stg_apply_level_jacobian", "stg_vcycle", "stg_smooth", "stg_prolongate", "stg_restrict",
+            "stg_apply_level_jacobian", "stg_vcycle", "stg_smooth", "stg_level_residual", "stg_prolongate", "stg_restrict",
             "stg_coarse_solve", "stg_gmres_solve", "stg_get_sizes", "stg_get_local_inverse", "stg_profile",
             "stg_profile_read", "stg_kernel_launches", "stg_invert_local_noalloc", "stg_newton_slab",
             "stg_slab_initial_guess", "stg_obstacle_forces", "stg_autotune", "stg_set_wait_limit", "stg_get_colour_variant",
@@ -89,6 +89,7 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
         "stg_apply_level_jacobian": (I, [P, I, P, P]),
         "stg_vcycle": (I, [P, P, P]),
         "stg_smooth": (I, [P, I, I, P, P]),
+        "stg_level_residual": (I, [P, I, P, P, P]),
         "stg_prolongate": (I, [P, I, P, P]),
         "stg_restrict": (I, [P, I, P, P]),
         "stg_coarse_solve": (I, [P, P, P]),
@@ -266,6 +267,13 @@ class Solver:
         x = self._dev(x).clone()
         self._call(self.lib.stg_smooth, level, sweeps, self._p(b), self._p(x))
         return x
+
+    def level_residual(self, level: int, b, x):
+        """b - J x on a level as the V-cycle computes it (in its precision)."""
+        b, x = self._dev(b), self._dev(x)
+        r = self.torch.empty_like(b)
+        self._call(self.lib.stg_level_residual, level, self._p(b), self._p(x), self._p(r))
+        return r
 
     def prolongate(self, level: int, xc, xf):
         xc = self._dev(xc)

@@ -192,6 +192,7 @@ struct LevelBufs {
   float *mk32 = nullptr, *ak32 = nullptr;  // Kronecker-split FP32 velocity rows (F32 form, levels >= 1, 2D)
   void *op_lin = nullptr, *op_oseen = nullptr;  // coefficients of the matrix-free FP64 operator: the option's, Oseen's
   const double* op_w = nullptr;  // velocity of the level's FP64 operator: w, or a Newton iterate's (then Oseen)
+  float* vd32 = nullptr;  // diagonals of the FP32 velocity blocks (F32 form, levels >= 1, 3D and order 4, k = 0, Oseen)
   float* w32 = nullptr;  // w and coefficients of the matrix-free FP32 residual (F32 form, levels >= 1, 3D and order 4)
   void* mf = nullptr;
   void* jinv = nullptr;
@@ -341,6 +342,7 @@ void linearise_internal(stg_ctx* c) {
     const long long nvp = L.g.n_cells * L.g.nloc * L.g.nt * L.g.dim * L.g.npd;
     convert(nvp, L.vp, L.vp32, s);
     convert(nvp, L.pv, L.pv32, s);
+    if (L.vd32) diagonal_blocks(L.g, L.nnzb, L.vv, L.vd32, s);
     if (L.mk32) kron_split(L.g, L.nnzb, L.vv, c->td, L.mk32, L.ak32, s);
   };
   for (int i = 0; i < nl; ++i) {
@@ -421,6 +423,9 @@ template <typename VT>
 void residual(stg_ctx* c, const LevelBufs& L, const VT* x, const VT* b, VT* r) {
   if (std::is_same<VT, float>::value && L.mf)
     residual_mf(L.g, L.mf, L.w32, (const float*)x, (const float*)b, c->mf_scr, (float*)r, c->st);
+  else if (std::is_same<VT, float>::value && L.vd32)
+    apply_operator_diag(L.g, L.rowptr, L.colidx, L.vd32, L.vp32, L.pv32, (const float*)x, (const float*)b, (float*)r,
+                        c->st);
   else if (std::is_same<VT, float>::value && L.mk32)
     apply_operator_kron(L.g, c->td, L.mk32, L.ak32, L.vp32, L.pv32, (const float*)x, (const float*)b,
                         (float*)r, c->st);
@@ -1009,9 +1014,9 @@ stg_status stg_setup(const stg_mesh* mesh, int k, double nu, double tau, const d
       const long long nvp = g.n_cells * g.nloc * g.nt * g.dim * g.npd;
       L.vp = dalloc<double>(c, nvp);
       L.pv = dalloc<double>(c, nvp);
-      if (!f64 && l > 0 && residual_mf_supported(g)) {
+      if (!f64 && l > 0 && residual_mf_supported(g, opt->linearisation == STG_NEWTON)) {
         L.w32 = dalloc<float>(c, g.nvel);
-        L.mf = dalloc<char>(c, (long long)residual_coef_bytes());
+        L.mf = dalloc<char>(c, (long long)residual_coef_bytes(g, 4));
       } else if (!f64 && l > 0) {
         L.vp32 = dalloc<float>(c, nvp);
         L.pv32 = dalloc<float>(c, nvp);
@@ -1020,14 +1025,16 @@ stg_status stg_setup(const stg_mesh* mesh, int k, double nu, double tau, const d
           // FP64 blocks as it gathers them: no FP32 copy of the dense blocks
           L.mk32 = dalloc<float>(c, L.nnzb);
           L.ak32 = dalloc<float>(c, L.nnzb * g.nt * g.dim * g.dim);
+        } else if ((g.dim == 3 || g.r == 4) && opt->linearisation == STG_OSEEN) {
+          L.vd32 = dalloc<float>(c, L.nnzb * g.NV);
         } else {
           L.vv32 = dalloc<float>(c, L.nnzb * g.NV * g.NV);
         }
       }
       L.w = dalloc<double>(c, g.nvel);
       if (operator_mf_preferred(g)) {
-        L.op_lin = dalloc<char>(c, (long long)residual_coef_bytes());
-        L.op_oseen = dalloc<char>(c, (long long)residual_coef_bytes());
+        L.op_lin = dalloc<char>(c, (long long)residual_coef_bytes(g, 8));
+        L.op_oseen = dalloc<char>(c, (long long)residual_coef_bytes(g, 8));
       }
       L.asm_tab = dalloc<double>(c, assemble_table_doubles(g.dim, k));
       L.vconst = dalloc<double>(c, L.nnzb * g.NV * g.NV);
@@ -1199,6 +1206,27 @@ stg_status stg_smooth(stg_ctx* c, int level, int sweeps, const double* b, double
       internal_to_cabi<float>(L.g, (const float*)L.x, x, c->st);
     }
     if (colour_kernel_timed_out(c->st)) throw Error{STG_ETIMEOUT, kColourTimeout};
+    return STG_OK;
+  } catch (const Error& e) {
+    return fail(c, e);
+  }
+}
+
+stg_status stg_level_residual(stg_ctx* c, int level, const double* b, const double* x, double* r) {
+  if (!c || !b || !x || !r || level < 1 || level >= (int)c->lv.size()) return STG_EINVAL;
+  try {
+    const LevelBufs& L = c->lv[level];
+    auto run = [&](auto tag) {
+      using VT = decltype(tag);
+      cabi_to_internal<VT>(L.g, b, (VT*)L.b, c->st);
+      cabi_to_internal<VT>(L.g, x, (VT*)L.x, c->st);
+      residual<VT>(c, L, (const VT*)L.x, (const VT*)L.b, (VT*)L.r);
+      internal_to_cabi<VT>(L.g, (const VT*)L.r, r, c->st);
+    };
+    if (vc64(c))
+      run(0.0);
+    else
+      run(0.f);
     return STG_OK;
   } catch (const Error& e) {
     return fail(c, e);

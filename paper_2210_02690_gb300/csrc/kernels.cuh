@@ -50,18 +50,24 @@ template <typename MT, typename VT>
 void apply_operator(const Geom& g, const int* rowptr, const int* colidx, const MT* vv, const MT* vp, const MT* pv,
                     const VT* x, const VT* b, VT* out, cudaStream_t st);
 
+// The same in FP32 from the diagonals of the velocity blocks, where the components do not couple (one Radau node,
+// Oseen, no obstacle): vd[slot][c], rounded from the FP64 blocks.
+void diagonal_blocks(const Geom& g, long long nnzb, const double* vv, float* vd, cudaStream_t st);
+void apply_operator_diag(const Geom& g, const int* rowptr, const int* colidx, const float* vd, const float* vp,
+                         const float* pv, const float* x, const float* b, float* out, cudaStream_t st);
+
 // The same in FP32 without a matrix (residual.cu), from the linearisation velocity w (FP32, internal
-// layout) and the coefficients that residual_coef writes to residual_coef_bytes() of device memory.
+// layout) and the coefficients that residual_coef writes to residual_coef_bytes(g, 4) of device memory.
 // scratch: residual_scratch(g) floats.
-bool residual_mf_supported(const Geom& g);
+bool residual_mf_supported(const Geom& g, bool newton);
 long long residual_scratch(const Geom& g);
-size_t residual_coef_bytes();
+size_t residual_coef_bytes(const Geom& g, size_t value);
 void residual_coef(const Geom& g, const TimeData& td, const AsmCoef& cf, void* dst, cudaStream_t st);
 void residual_mf(const Geom& g, const void* coef, const float* w, const float* x, const float* b, float* scratch,
                  float* out, cudaStream_t st);
 
 // The FP64 operator without a matrix (3D, residual64.cu): out = b - J x, or J x (b null), at linearisation velocity w (FP64,
-// internal layout); coef as above, scratch: residual_scratch(g) doubles.
+// internal layout); coef: residual_coef_bytes(g, 8) bytes from operator_coef, scratch: residual_scratch(g) doubles.
 bool operator_mf_preferred(const Geom& g);
 void operator_coef(const Geom& g, const TimeData& td, const AsmCoef& cf, void* dst, cudaStream_t st);
 void operator_mf(const Geom& g, const void* coef, const double* w, const double* x, const double* b, double* scratch,

@@ -1,17 +1,21 @@
-// J x and b - J x without a matrix: the FP32 V-cycle's residual in 3D and for order 4 (residual.cu; the 2D order-2 levels
-// use vanka.cu's split rows) and the FP64 operator in 3D (residual64.cu).
+// J x and b - J x without a matrix: the FP32 V-cycle's residual in 3D and for order 4 from two Radau nodes on (residual.cu;
+// the other levels use vanka.cu's rows) and the FP64 operator in 3D (residual64.cu).
 //
 // The slab operator (Eq. (3.3) with D_ab and B_ab of Eq. (2.1), (2.2)) applied cell by cell by sum
 // factorisation: the nodal values of a cell are interpolated to its Gauss points one direction at a
 // time, differentiated there by the 1D collocation derivative, combined with the linearisation
 // velocity at the points, and taken back by the transposed steps.  One thread holds one component
 // (Radau node a, direction c) of one cell; the components of a cell exchange their values at the
-// Gauss points through shared memory (time coupling, convection, Newton's term).  Everything is read
-// from nodal vectors, so a residual moves a few vectors where the assembled operator moved
-// 4 (1 + (k+1) d^2) bytes per node pair in 2D and 4 ((k+1) d)^2 in 3D.
+// Gauss points through shared memory (time coupling, convection, Newton's term).  The velocity-pressure
+// coupling is a small table per Radau node, component and set of Dirichlet faces, integrated in FP64 and
+// rounded once, as an assembled block is: summed over the Gauss points in FP32 the pressure rows of order 4
+// had twice an assembled row's rounding error.  Everything else is read from nodal vectors, so a residual
+// moves a few vectors where the assembled operator moved 4 (1 + (k+1) d^2) bytes per node pair in 2D and
+// 4 ((k+1) d)^2 in 3D.
 #pragma once
 
 #include <algorithm>
+#include <cstring>
 
 #include "common.cuh"
 #include "kernels.cuh"
@@ -29,6 +33,7 @@ struct Ref {
   T L[M][M];           // Lagrange function of node l at Gauss point q: [q][l]
   T G[M][M];           // derivative at Gauss point q of the Lagrange function of Gauss point p: [q][p]
   T DN[2][M];          // derivative at -1 and +1 of the Lagrange function of node l
+  T MM[M][M];          // integral of the product of the Lagrange functions of nodes l and m
 };
 
 template <int DIM, int M, typename T>
@@ -81,6 +86,9 @@ constexpr Ref<DIM, M, T> make_ref() {
       }
       r.DN[s][l] = d;
     }
+  for (int l = 0; l < M; ++l)
+    for (int m = 0; m < M; ++m)
+      for (int q = 0; q < M; ++q) r.MM[l][m] += r.w[q] * r.L[q][l] * r.L[q][m];
   Ref<DIM, M, T> o{};
   for (int i = 0; i < M; ++i) {
     o.x[i] = (T)r.x[i];
@@ -88,6 +96,7 @@ constexpr Ref<DIM, M, T> make_ref() {
     for (int j = 0; j < M; ++j) {
       o.L[i][j] = (T)r.L[i][j];
       o.G[i][j] = (T)r.G[i][j];
+      o.MM[i][j] = (T)r.MM[i][j];
     }
     for (int k = 0; k < 2; ++k) o.DN[k][i] = (T)r.DN[k][i];
   }
@@ -101,11 +110,11 @@ template <int DIM, int M, typename T>
 __constant__ Ref<DIM, M, T> c_ref = make_ref<DIM, M, T>();
 
 // Pressure function m of P_{r-1}^disc at reference coordinates c.
-template <int DIM, int M, typename T>
-__device__ __forceinline__ T pressure_fn(int m, const T* c) {
-  if (m == 0) return (T)1;
+template <int M>
+__device__ __forceinline__ double pressure_fn(int m, const double* c) {
+  if (m == 0) return 1.0;
   if (M == 3 || m <= 2) return c[m - 1];
-  const T x = c[0], y = c[1];
+  const double x = c[0], y = c[1];
   return m == 3 ? x * x : m == 4 ? x * y : m == 5 ? y * y : m == 6 ? x * x * x : m == 7 ? x * x * y : m == 8 ? x * y * y
                                                                                                         : y * y * y;
 }
@@ -121,17 +130,106 @@ struct MfCoef {
   int newton;
 };
 
+// Pressure coefficients of a cell and Radau node, and the same padded to whole 16-byte loads of the table.
+template <int M>
+constexpr int kNP = M == 3 ? 4 : 10;  // M == 3: 3D
+template <int M>
+constexpr int kNPP = M == 3 ? 4 : 12;
+
+// Entry (a, faces, c, i, m): pressure row m of Radau node a against component c at node i of a cell with these
+// Dirichlet faces (bit 2 e + side).  The velocity rows take the negative transpose.
+template <int DIM, int M, typename T>
+__global__ void __launch_bounds__(128) pressure_table(int count, MfCoef<double> cf, T* __restrict__ table) {
+  const Ref<DIM, M, double>& R = c_ref<DIM, M, double>;
+  constexpr int N = ipow(M, DIM), NCLS = 1 << (2 * DIM);
+  const int t = blockIdx.x * 128 + threadIdx.x;
+  if (t >= count) return;
+  const int m = t % kNPP<M>, i = t / kNPP<M> % N, c = t / (kNPP<M> * N) % DIM;
+  const int faces = t / (kNPP<M> * N * DIM) % NCLS, a = t / (kNPP<M> * N * DIM * NCLS);
+  if (m >= kNP<M>) {
+    table[t] = (T)0;
+    return;
+  }
+  const int in[3] = {i % M, i / M % M, i / (M * M)};
+  double sum = 0.0;
+  for (int q = 0; q < N; ++q) {
+    const int qn[3] = {q % M, q / M % M, q / (M * M)};
+    double v = 0.0, x[3];
+    for (int p = 0; p < M; ++p) v += R.G[qn[c]][p] * R.L[p][in[c]];
+    for (int e = 0; e < DIM; ++e) {
+      x[e] = R.x[qn[e]];
+      v *= e == c ? R.w[qn[e]] : R.w[qn[e]] * R.L[qn[e]][in[e]];
+    }
+    sum += v * pressure_fn<M>(m, x);
+  }
+  for (int side = 0; side < 2; ++side) {
+    if (!(faces >> (2 * c + side) & 1) || in[c] != (side ? M - 1 : 0)) continue;
+    const int e1 = c == 0 ? 1 : 0, e2 = c == 2 ? 1 : 2;
+    for (int q = 0; q < N / M; ++q) {
+      const int q1 = q % M, q2 = q / M;
+      double x[3], v = R.w[q1] * R.L[q1][in[e1]];
+      x[c] = side ? 1.0 : -1.0;
+      x[e1] = R.x[q1];
+      if (DIM == 3) {
+        x[e2] = R.x[q2];
+        v *= R.w[q2] * R.L[q2][in[e2]];
+      }
+      sum -= (side ? 1.0 : -1.0) * v * pressure_fn<M>(m, x);
+    }
+  }
+  table[t] = (T)(cf.sa[a] * cf.sc[c] * sum);
+}
+
+template <int M, typename T>
+__device__ __forceinline__ void load_table_row(const T* __restrict__ p, T (&t)[kNPP<M>]) {
+  constexpr int V = 16 / sizeof(T);
+#pragma unroll
+  for (int j = 0; j < kNPP<M> / V; ++j) {
+    const int4 u = __ldg(reinterpret_cast<const int4*>(p) + j);
+    memcpy(&t[V * j], &u, 16);
+  }
+}
+
+// A component's part of a cell's pressure rows from its nodal values V; table: the component's rows.
+template <int M, int N, typename T>
+__device__ __forceinline__ void pressure_rows(const T* __restrict__ table, const T (&V)[N], T (&pp)[kNP<M>]) {
+#pragma unroll
+  for (int m = 0; m < kNP<M>; ++m) pp[m] = (T)0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    T t[kNPP<M>];
+    load_table_row<M, T>(table + i * kNPP<M>, t);
+#pragma unroll
+    for (int m = 0; m < kNP<M>; ++m) pp[m] += t[m] * V[i];
+  }
+}
+
+// The pressure's part of the component's nodal rows, added to V.
+template <int M, int N, typename T>
+__device__ __forceinline__ void add_pressure(const T* __restrict__ table, const T (&p)[kNP<M>], T (&V)[N]) {
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    T t[kNPP<M>];
+    load_table_row<M, T>(table + i * kNPP<M>, t);
+#pragma unroll
+    for (int m = 0; m < kNP<M>; ++m) V[i] -= t[m] * p[m];
+  }
+}
+
 // One cell, component (a, c): on entry V = nodal values of x, W of the linearisation velocity; on
-// return V holds the cell's contribution to the nodal rows and pp[m] this component's part of
-// the pressure rows.  sv, sw: Gauss-point values of all components, [a DIM + c][point][lane].  faces: the
-// cell's Dirichlet faces; nodal(i): the value of x at node i once more, for them.  Contains one barrier of the
-// CTA.
+// return V holds the cell's contribution to the nodal rows, without the pressure's.  sv, sw: Gauss-point
+// values of all components, [a DIM + c][point][lane].  on: the lane has a cell; faces: its Dirichlet faces;
+// nodal(i, b): the value of x at node i and Radau node b once more.  Contains one barrier of the CTA.
+//
+// The time coupling of order 4 goes from nodes to nodes by the 1D mass matrices: through the Gauss points, with
+// four factors of L, its velocity rows had up to 1.2 times the rounding error of assembled ones (k = 1, Oseen; the
+// mass term is the largest there).  For order 2 the Gauss points round less (1D weights 1/15 to 16/15).
 template <int DIM, int M, int NT, typename T, typename Nodal>
 __device__ __forceinline__ void cell_operator(const MfCoef<T>& cf, int a, int c, unsigned faces, T (&V)[ipow(M, DIM)],
-                                              T (&W)[ipow(M, DIM)], const T* __restrict__ p, T* sv, T* sw, int lane,
-                                              T* pp, Nodal nodal) {
+                                              T (&W)[ipow(M, DIM)], T* sv, T* sw, int lane, bool on, Nodal nodal) {
   const Ref<DIM, M, T>& R = c_ref<DIM, M, T>;
-  constexpr int N = ipow(M, DIM), NP = M == 3 ? DIM + 1 : 10;
+  constexpr int N = ipow(M, DIM);
+  constexpr bool kNodalMass = M == 5;
   auto interp = [&](T(&u)[N]) {
 #pragma unroll
     for (int e = 0; e < DIM; ++e) {
@@ -164,14 +262,15 @@ __device__ __forceinline__ void cell_operator(const MfCoef<T>& cf, int a, int c,
   const T sa = cf.sa[a];
 #pragma unroll
   for (int q = 0; q < N; ++q) {
-    T t = cf.time[a][0] * sv[(c * N + q) * 32 + lane];
+    T t = (T)0;
+    if constexpr (!kNodalMass) {
+      t = cf.time[a][0] * sv[(c * N + q) * 32 + lane];
 #pragma unroll
-    for (int b = 1; b < NT; ++b) t += cf.time[a][b] * sv[((b * DIM + c) * N + q) * 32 + lane];
+      for (int b = 1; b < NT; ++b) t += cf.time[a][b] * sv[((b * DIM + c) * N + q) * 32 + lane];
+    }
     val[q] = t;
     res[q] = (T)0;
   }
-#pragma unroll
-  for (int m = 0; m < NP; ++m) pp[m] = (T)0;
 #pragma unroll
   for (int e = 0; e < DIM; ++e) {
     const int st = e == 0 ? 1 : e == 1 ? M : M * M;
@@ -195,19 +294,7 @@ __device__ __forceinline__ void cell_operator(const MfCoef<T>& cf, int a, int c,
           add += sv[((a * DIM + e) * N + id) * 32 + lane] * (dw * (sce * sa));
         }
         val[id] += add;
-        const T wt = R.wt[id];
-        T fl = cf.nu * dv;
-        if (e == c) {
-          const T pt[3] = {R.x[id % M], R.x[(id / M) % M], DIM == 3 ? R.x[id / (M * M) % M] : (T)0};
-          T pr = p[0];
-#pragma unroll
-          for (int m = 1; m < NP; ++m) pr += pressure_fn<DIM, M, T>(m, pt) * p[m];
-          fl -= sa * pr;
-          const T wd = wt * dv;
-#pragma unroll
-          for (int m = 0; m < NP; ++m) pp[m] += pressure_fn<DIM, M, T>(m, pt) * wd;
-        }
-        F[q] = wt * sce * fl;
+        F[q] = R.wt[id] * sce * (cf.nu * dv);
       }
 #pragma unroll
       for (int q = 0; q < M; ++q)
@@ -240,6 +327,34 @@ __device__ __forceinline__ void cell_operator(const MfCoef<T>& cf, int a, int c,
   }
 #pragma unroll
   for (int q = 0; q < N; ++q) V[q] = res[q];
+  if constexpr (kNodalMass) {
+    T t[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      t[i] = (T)0;
+#pragma unroll
+      for (int b = 0; b < NT; ++b) t[i] += cf.time[a][b] * (on ? nodal(i, b) : (T)0);
+    }
+#pragma unroll
+    for (int e = 0; e < DIM; ++e) {
+      const int st = e == 0 ? 1 : e == 1 ? M : M * M;
+#pragma unroll
+      for (int ln = 0; ln < N / M; ++ln) {
+        const int o = (ln / st) * st * M + ln % st;
+        T u[M];
+#pragma unroll
+        for (int q = 0; q < M; ++q) {
+          u[q] = R.MM[q][0] * t[o];
+#pragma unroll
+          for (int l = 1; l < M; ++l) u[q] += R.MM[q][l] * t[o + l * st];
+        }
+#pragma unroll
+        for (int q = 0; q < M; ++q) t[o + q * st] = u[q];
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) V[i] += t[i];
+  }
   // Nitsche's terms of the Dirichlet faces, in nodal values: the penalty gamma2 / h is large against the other
   // terms, and only the face's own rows may carry its rounding
   if (faces) {
@@ -275,7 +390,7 @@ __device__ __forceinline__ void cell_operator(const MfCoef<T>& cf, int a, int c,
         dn[k] = (T)0;
 #pragma unroll
         for (int l = 0; l < M; ++l) {
-          const T u = nodal(o + l * st);
+          const T u = nodal(o + l * st, a);
           dn[k] += R.DN[s0][l] * u;
           if (l == (s0 ? M - 1 : 0)) tr[k] = u;
         }
@@ -288,16 +403,7 @@ __device__ __forceinline__ void cell_operator(const MfCoef<T>& cf, int a, int c,
         T wt = sa * cf.sc[e0] * R.w[t0];
         if (DIM == 3) wt *= R.w[t1];
         T A = cf.g1[e0] * tr[k] - cf.nu * sn * dn[k];
-        if (e0 == c) {
-          const T pt[3] = {e0 == 0 ? ns : R.x[t0], e0 == 1 ? ns : (e0 == 0 ? R.x[t0] : R.x[t1]), e0 == 2 ? ns : R.x[t1]};
-          T pr = p[0];
-#pragma unroll
-          for (int m = 1; m < NP; ++m) pr += pressure_fn<DIM, M, T>(m, pt) * p[m];
-          A += cf.g2[e0] * tr[k] + ns * pr;
-          const T wd = -ns * wt * tr[k];
-#pragma unroll
-          for (int m = 0; m < NP; ++m) pp[m] += pressure_fn<DIM, M, T>(m, pt) * wd;
-        }
+        if (e0 == c) A += cf.g2[e0] * tr[k];
         dn[k] = -cf.nu * sn * tr[k] * wt;
         tr[k] = A * wt;
       }
@@ -339,12 +445,13 @@ __device__ __forceinline__ unsigned cell_faces(const Geom& g, int cx, int cy, in
 // kept from the previous step (the row below the owned ones is computed for that alone).  Bound by FP32
 // issue; the repeated column and row cost 32/31 and (ty + 1)/ty.
 template <int M, int NT, typename T>
-__global__ void __launch_bounds__(64 * NT) mf_residual2d(Geom g, const MfCoef<T>* __restrict__ cfp, const T* __restrict__ w,
+__global__ void __launch_bounds__(64 * NT, NT == 2 ? 3 : 2) mf_residual2d(Geom g, const MfCoef<T>* __restrict__ cfp,
+                                                        const T* __restrict__ table, const T* __restrict__ w,
                                                         const T* __restrict__ x, const T* __restrict__ b,
                                                         T* __restrict__ out, int ty) {
   pdl_wait();
   const MfCoef<T>& cf = *cfp;
-  constexpr int N = M * M, R = M - 1, NV = 2 * NT, NP = M == 3 ? 3 : 10;
+  constexpr int N = M * M, R = M - 1, NV = 2 * NT, NP = kNP<M>;
   extern __shared__ __align__(16) unsigned char mf_smem[];
   T* sv = reinterpret_cast<T*>(mf_smem);
   T* sw = sv + NV * N * 32;
@@ -378,11 +485,16 @@ __global__ void __launch_bounds__(64 * NT) mf_residual2d(Geom g, const MfCoef<T>
 #pragma unroll
       for (int m = 0; m < NP; ++m) P[m] = pc[m];
     }
-    cell_operator<2, M, NT, T>(cf, a, c, dead ? 0u : cell_faces<2>(g, cx, cy, 0), V, W, P, sv, sw, lane, pp,
-                               [&](int i) { return x[n0 + ((long long)(i / M) * g.nn[0] + i % M) * NV]; });
+    const unsigned faces = dead ? 0u : cell_faces<2>(g, cx, cy, 0);
+    const T* rows_c = table + ((a * 16 + faces) * 2 + c) * (N * kNPP<M>);
+    pressure_rows<M, N, T>(rows_c, V, pp);
+    __syncthreads();  // the cell row below has been read from shared memory
 #pragma unroll
     for (int m = 0; m < NP; ++m) sp[(v * NP + m) * 32 + lane] = pp[m];
-    __syncthreads();
+    cell_operator<2, M, NT, T>(cf, a, c, faces, V, W, sv, sw, lane, !dead, [&](int i, int b_) {
+      return x[n0 + ((long long)(i / M) * g.nn[0] + i % M) * NV + 2 * (b_ - a)];
+    });
+    add_pressure<M, N, T>(rows_c, P, V);
     const bool write = cy >= y0;
     if (write && owned) {
       const long long o0 = g.nvel + ((long long)cy * g.n[0] + cx) * (NT * NP) + a * NP;
@@ -420,12 +532,13 @@ __global__ void __launch_bounds__(64 * NT) mf_residual2d(Geom g, const MfCoef<T>
 // 3D: the cells' contributions E[(v, node)][cell] and the pressure rows, one thread per (cell, component);
 // then mf_nodes3d sums each node's cells.  E (4 * 27 bytes per cell and component) mostly stays in L2.
 template <int NT, typename T>
-__global__ void __launch_bounds__(96 * NT) mf_cells3d(Geom g, const MfCoef<T>* __restrict__ cfp, const T* __restrict__ w,
+__global__ void __launch_bounds__(96 * NT) mf_cells3d(Geom g, const MfCoef<T>* __restrict__ cfp,
+                                                     const T* __restrict__ table, const T* __restrict__ w,
                                                      const T* __restrict__ x, const T* __restrict__ b,
                                                      T* __restrict__ E, T* __restrict__ out) {
   pdl_wait();
   const MfCoef<T>& cf = *cfp;
-  constexpr int N = 27, NV = 3 * NT, NP = 4;
+  constexpr int N = 27, NV = 3 * NT, NP = kNP<3>;
   extern __shared__ __align__(16) unsigned char mf_smem[];
   T* sv = reinterpret_cast<T*>(mf_smem);
   T* sw = sv + NV * N * 32;
@@ -456,16 +569,16 @@ __global__ void __launch_bounds__(96 * NT) mf_cells3d(Geom g, const MfCoef<T>* _
   auto node = [&](int i) {
     return n0 + (i % 3 + (long long)g.nn[0] * ((i / 3) % 3 + (long long)g.nn[1] * (i / 9))) * NV;
   };
-  cell_operator<3, 3, NT, T>(cf, a, c, on ? cell_faces<3>(g, cx, cy, cz) : 0u, V, W, P, sv, sw, lane, pp,
-                             [&](int i) { return x[node(i)]; });
+  const unsigned faces = on ? cell_faces<3>(g, cx, cy, cz) : 0u;
+  const T* rows_c = table + ((a * 64 + faces) * 3 + c) * (N * kNPP<3>);
+  pressure_rows<3, N, T>(rows_c, V, pp);
 #pragma unroll
   for (int m = 0; m < NP; ++m) sp[(v * NP + m) * 32 + lane] = pp[m];
+  cell_operator<3, 3, NT, T>(cf, a, c, faces, V, W, sv, sw, lane, on, [&](int i, int) { return x[node(i)]; });
+  add_pressure<3, N, T>(rows_c, P, V);
   if (on) {
 #pragma unroll
     for (int i = 0; i < N; ++i) E[((long long)v * N + i) * g.n_cells + cell] = V[i];
-  }
-  __syncthreads();
-  if (on) {
     const long long o0 = g.nvel + cell * (NT * NP) + a * NP;
     for (int m = c; m < NP; m += 3) {
       T s = (T)0;
@@ -519,46 +632,47 @@ MfCoef<T> coefficients(const Geom& g, const TimeData& td, const AsmCoef& cf) {
 // At least two CTAs per SM of the 152 where the mesh has them, at most 16 rows a CTA.
 constexpr int kMinCtas = 304;
 
+template <int DIM, int M, typename T>
+constexpr int pressure_table_values(int nt) {
+  return nt * (1 << (2 * DIM)) * DIM * ipow(M, DIM) * kNPP<M>;
+}
+// The coefficients, then the pressure table.
+constexpr size_t kTableOffset = (sizeof(MfCoef<double>) + 15) / 16 * 16;
+template <typename T>
+const T* table_of(const void* coef) {
+  return reinterpret_cast<const T*>(static_cast<const char*>(coef) + kTableOffset);
+}
+
 template <int M, int NT, typename T>
-void run2d(const Geom& g, const MfCoef<T>* m, const T* w, const T* x, const T* b, T* out, cudaStream_t st) {
-  constexpr int NV = 2 * NT, NP = M == 3 ? 3 : 10;
-  constexpr size_t smem = sizeof(T) * 32 * NV * (2 * M * M + NP);
+void run2d(const Geom& g, const void* coef, const T* w, const T* x, const T* b, T* out, cudaStream_t st) {
+  constexpr int NV = 2 * NT;
+  constexpr size_t smem = sizeof(T) * 32 * NV * (2 * M * M + kNP<M>);
   if (smem > 48 * 1024)
     STG_CUDA_OK(cudaFuncSetAttribute(mf_residual2d<M, NT, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const int nbx = (g.n[0] + 30) / 31;
   const int ty = std::max(1, std::min(16, (int)((long long)nbx * g.n[1] / kMinCtas)));
-  launch_k(mf_residual2d<M, NT, T>, dim3(nbx, (g.n[1] + ty - 1) / ty), dim3(32, NV), smem, st, g, m, w, x, b, out, ty);
+  launch_k(mf_residual2d<M, NT, T>, dim3(nbx, (g.n[1] + ty - 1) / ty), dim3(32, NV), smem, st, g, (const MfCoef<T>*)coef,
+           table_of<T>(coef), w, x, b, out, ty);
 }
 
 template <int NT, typename T>
-void run3d(const Geom& g, const MfCoef<T>* m, const T* w, const T* x, const T* b, T* E, T* out, cudaStream_t st) {
-  constexpr size_t smem = sizeof(T) * 32 * (3 * NT) * (2 * 27 + 4);
+void run3d(const Geom& g, const void* coef, const T* w, const T* x, const T* b, T* E, T* out, cudaStream_t st) {
+  constexpr size_t smem = sizeof(T) * 32 * (3 * NT) * (2 * 27 + kNP<3>);
   if (smem > 48 * 1024)
     STG_CUDA_OK(cudaFuncSetAttribute(mf_cells3d<NT, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  launch_k(mf_cells3d<NT, T>, grid_for(g.n_cells, 32), dim3(32, 3 * NT), smem, st, g, m, w, x, b, E, out);
+  launch_k(mf_cells3d<NT, T>, grid_for(g.n_cells, 32), dim3(32, 3 * NT), smem, st, g, (const MfCoef<T>*)coef,
+           table_of<T>(coef), w, x, b, E, out);
   launch_k(mf_nodes3d<T>, dim3((g.nn[0] + 31) / 32, g.nn[1], g.nn[2]), dim3(32, 3 * NT), 0, st, g, E, b, out);
 }
 
-template <int M, typename T>
-void dispatch2d(const Geom& g, const MfCoef<T>* m, const T* w, const T* x, const T* b, T* out, cudaStream_t st) {
-  switch (g.nt) {
-    case 1: return run2d<M, 1, T>(g, m, w, x, b, out, st);
-    case 2: return run2d<M, 2, T>(g, m, w, x, b, out, st);
-    default: return run2d<M, 3, T>(g, m, w, x, b, out, st);
-  }
-}
-template <typename T>
-void dispatch3d(const Geom& g, const MfCoef<T>* m, const T* w, const T* x, const T* b, T* E, T* out, cudaStream_t st) {
-  switch (g.nt) {
-    case 1: return run3d<1, T>(g, m, w, x, b, E, out, st);
-    case 2: return run3d<2, T>(g, m, w, x, b, E, out, st);
-    default: return run3d<3, T>(g, m, w, x, b, E, out, st);
-  }
-}
-template <typename T>
+template <int DIM, int M, typename T>
 void upload_coefficients(const Geom& g, const TimeData& td, const AsmCoef& cf, void* dst, cudaStream_t st) {
   const MfCoef<T> m = coefficients<T>(g, td, cf);
   STG_CUDA_OK(cudaMemcpyAsync(dst, &m, sizeof(m), cudaMemcpyHostToDevice, st));
+  const int count = pressure_table_values<DIM, M, T>(g.nt);
+  pressure_table<DIM, M, T><<<(count + 127) / 128, 128, 0, st>>>(count, coefficients<double>(g, td, cf),
+                                                                const_cast<T*>(table_of<T>(dst)));
+  STG_LAUNCH_OK();
 }
 
 }  // namespace

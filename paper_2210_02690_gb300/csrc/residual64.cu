@@ -9,13 +9,17 @@ namespace stg {
 bool operator_mf_preferred(const Geom& g) { return g.dim == 3; }
 
 void operator_coef(const Geom& g, const TimeData& td, const AsmCoef& cf, void* dst, cudaStream_t st) {
-  upload_coefficients<double>(g, td, cf, dst, st);
+  upload_coefficients<3, 3, double>(g, td, cf, dst, st);
 }
 
 void operator_mf(const Geom& g, const void* coef, const double* w, const double* x, const double* b, double* scratch,
                  double* out, cudaStream_t st) {
   if (g.dim != 3) throw Error{STG_EINVAL, "no matrix-free FP64 operator in 2D"};
-  dispatch3d<double>(g, (const MfCoef<double>*)coef, w, x, b, scratch, out, st);
+  switch (g.nt) {
+    case 1: return run3d<1, double>(g, coef, w, x, b, scratch, out, st);
+    case 2: return run3d<2, double>(g, coef, w, x, b, scratch, out, st);
+    default: return run3d<3, double>(g, coef, w, x, b, scratch, out, st);
+  }
 }
 
 }  // namespace stg

@@ -38,7 +38,9 @@ __device__ __forceinline__ void op_pres_row(const Geom& g, const MT* __restrict_
 // a warp do not diverge, and with NT known the terms of a slot are loaded together.
 // Whole steps: 256^2 k = 3 42.1 -> 40.1 ms, 256^2 k = 2 21.9 -> 20.4, 704x128 FP64 form 70.3 -> 67.9,
 // 8x8 k = 0 3.41 -> 3.02 (latency), same bits.
-template <int DIM, int NT, typename MT, typename VT>
+// DIAG (one Radau node, Oseen, no obstacle): the components do not couple either, and vv holds the DIM diagonal values
+// of a block alone.
+template <int DIM, int NT, typename MT, typename VT, bool DIAG = false>
 __global__ void __launch_bounds__(256) op_rows(Geom g, const int* __restrict__ rowptr, const int* __restrict__ colidx,
                                                const MT* __restrict__ vv, const MT* __restrict__ vp,
                                                const MT* __restrict__ pv, const VT* __restrict__ x,
@@ -49,7 +51,8 @@ __global__ void __launch_bounds__(256) op_rows(Geom g, const int* __restrict__ r
     if (t < g.N) op_pres_row<DIM, MT, VT>(g, pv, x, b, out, t - g.nvel);
     return;
   }
-  constexpr int NV = DIM * NT, NZ = NT + DIM - 1;
+  static_assert(!DIAG || NT == 1, "several Radau nodes couple");
+  constexpr int NV = DIM * NT, NZ = DIAG ? 1 : NT + DIM - 1;
   const long long node = t / NV;
   const int row = (int)(t - node * NV);
   VT acc = 0;
@@ -58,11 +61,11 @@ __global__ void __launch_bounds__(256) op_rows(Geom g, const int* __restrict__ r
 #pragma unroll
   for (int k = 0; k < NZ; ++k) {
     const int ra = row / DIM, rc = row % DIM;
-    off[k] = k < ra ? k * DIM + rc : k < ra + DIM ? ra * DIM + k - ra : (k - DIM + 1) * DIM + rc;
+    off[k] = DIAG ? row : k < ra ? k * DIM + rc : k < ra + DIM ? ra * DIM + k - ra : (k - DIM + 1) * DIM + rc;
   }
 #pragma unroll 4
   for (int blk = b0; blk < b1; ++blk) {
-    const MT* vals = vv + (long long)blk * NV * NV + (long long)row * NV;
+    const MT* vals = vv + (long long)blk * (DIAG ? NV : NV * NV) + (DIAG ? 0 : row * NV);
     const VT* xc = x + (long long)colidx[blk] * NV;
 #pragma unroll
     for (int k = 0; k < NZ; ++k) acc += (VT)vals[off[k]] * xc[off[k]];
@@ -90,6 +93,17 @@ __global__ void __launch_bounds__(256) op_rows(Geom g, const int* __restrict__ r
         for (int m = 0; m < npd; ++m) acc += (VT)q[m] * p[m];
       }
   out[t] = b ? b[t] - acc : acc;
+}
+
+// The diagonals of the velocity blocks, rounded to FP32.
+__global__ void __launch_bounds__(256) diagonal_blocks_kernel(long long nnzb, int NV, const double* __restrict__ vv,
+                                                             float* __restrict__ vd) {
+  pdl_wait();
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= nnzb * NV) return;
+  const long long blk = t / NV;
+  const int i = (int)(t - blk * NV);
+  vd[t] = (float)vv[(blk * NV + i) * NV + i];
 }
 
 // ------------------------------------------------------------------ Kronecker-split FP32 rows (2D)
@@ -1184,7 +1198,7 @@ void apply_operator(const Geom& g, const int* rowptr, const int* colidx, const M
                     const VT* x, const VT* b, VT* out, cudaStream_t st) {
   const unsigned grid = grid_for(g.N, 256);
   if constexpr (sizeof(MT) == 4) {
-    // the other FP32 levels take the Kronecker split (2D) or no matrix (3D, order 4)
+    // the other FP32 levels take the Kronecker split (2D order 2), the diagonals or no matrix (3D; order 4)
     if (g.dim != 2 || g.nt != 1) throw Error{STG_EINVAL, "no assembled FP32 operator on this level"};
     launch_k(op_rows<2, 1, MT, VT>, grid, 256, 0, st, g, rowptr, colidx, vv, vp, pv, x, b, out);
   } else if (g.dim == 2) {
@@ -1202,6 +1216,20 @@ void apply_operator(const Geom& g, const int* rowptr, const int* colidx, const M
       default: launch_k(op_rows<3, 3, MT, VT>, grid, 256, 0, st, g, rowptr, colidx, vv, vp, pv, x, b, out); break;
     }
   }
+}
+
+void diagonal_blocks(const Geom& g, long long nnzb, const double* vv, float* vd, cudaStream_t st) {
+  launch_k(diagonal_blocks_kernel, grid_for(nnzb * g.NV, 256), 256, 0, st, nnzb, g.NV, vv, vd);
+}
+
+void apply_operator_diag(const Geom& g, const int* rowptr, const int* colidx, const float* vd, const float* vp,
+                         const float* pv, const float* x, const float* b, float* out, cudaStream_t st) {
+  if (g.nt != 1) throw Error{STG_EINVAL, "diagonal velocity blocks need a single Radau node"};
+  const unsigned grid = grid_for(g.N, 256);
+  if (g.dim == 2)
+    launch_k(op_rows<2, 1, float, float, true>, grid, 256, 0, st, g, rowptr, colidx, vd, vp, pv, x, b, out);
+  else
+    launch_k(op_rows<3, 1, float, float, true>, grid, 256, 0, st, g, rowptr, colidx, vd, vp, pv, x, b, out);
 }
 
 bool kron_supported(const Geom& g) { return g.dim == 2 && g.r == 2 && g.nt >= 2 && g.nt <= 5; }

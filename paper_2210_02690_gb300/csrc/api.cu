@@ -190,8 +190,8 @@ struct LevelBufs {
   float *vv32 = nullptr, *vp32 = nullptr, *pv32 = nullptr;
   double* vconst = nullptr;  // the w = 0 assembly (time coupling, viscous, Nitsche), built once
   float *mk32 = nullptr, *ak32 = nullptr;  // Kronecker-split FP32 velocity rows (F32 form, levels >= 1, 2D)
-  void *op_lin = nullptr, *op_oseen = nullptr;  // coefficients of the matrix-free FP64 operator: the option's, Oseen's
-  const double* op_w = nullptr;  // velocity of the level's FP64 operator: w, or a Newton iterate's (then Oseen)
+  void* op = nullptr;      // coefficients of the matrix-free FP64 operator (3D, levels >= 1)
+  double* op_w = nullptr;  // and its velocity: w, on the finest level a copy of w or of a Newton iterate's (then Oseen)
   float* vd32 = nullptr;  // diagonals of the FP32 velocity blocks (F32 form, levels >= 1, 3D and order 4, k = 0, Oseen)
   float* w32 = nullptr;  // w and coefficients of the matrix-free FP32 residual (F32 form, levels >= 1, 3D and order 4)
   void* mf = nullptr;
@@ -313,16 +313,23 @@ void assemble_constant(stg_ctx* c) {
     STG_CUDA_OK(cudaMemcpyAsync(L.vconst, L.vv, sizeof(double) * L.nnzb * L.g.NV * L.g.NV,
                                 cudaMemcpyDeviceToDevice, c->st));
     if (L.mf) residual_coef(L.g, c->td, cf, L.mf, c->st);
-    if (L.op_lin) operator_coef(L.g, c->td, cf, L.op_lin, c->st);
-    if (L.op_oseen) operator_coef(L.g, c->td, cf0, L.op_oseen, c->st);
+    if (L.op) operator_coef(L.g, c->td, cf, L.op, c->st);
   }
+}
+
+// The finest level's matrix-free FP64 operator at the velocity part of X (internal layout), in place: the captured
+// V-cycle and every other user of the operator see it.
+void set_operator(stg_ctx* c, const double* X, bool newton) {
+  LevelBufs& F = c->lv.back();
+  STG_CUDA_OK(cudaMemcpyAsync(F.op_w, X, sizeof(double) * F.g.nvel, cudaMemcpyDeviceToDevice, c->st));
+  operator_set_newton(F.op, newton, c->st);
 }
 
 // Assemble every level for the finest-level linearisation velocity in F.w (internal
 // layout), invert the local matrices, factor the coarse system.
 void linearise_internal(stg_ctx* c) {
   const int nl = (int)c->lv.size();
-  for (LevelBufs& L : c->lv) L.op_w = L.w;
+  if (c->lv.back().op) set_operator(c, c->lv.back().w, c->opt.linearisation == STG_NEWTON);
   for (int l = nl - 1; l > 0; --l) inject_w(c->lv[l - 1].g, c->lv[l].g, c->lv[l].w, c->lv[l - 1].w, c->st);
   AsmCoef cf{c->nu, c->tau, c->opt.gamma1, c->opt.gamma2, c->opt.linearisation == STG_NEWTON ? 1 : 0};
   STG_CUDA_OK(cudaMemsetAsync(c->status, 0, sizeof(int) * 4, c->st));
@@ -429,17 +436,17 @@ void residual(stg_ctx* c, const LevelBufs& L, const VT* x, const VT* b, VT* r) {
   else if (std::is_same<VT, float>::value && L.mk32)
     apply_operator_kron(L.g, c->td, L.mk32, L.ak32, L.vp32, L.pv32, (const float*)x, (const float*)b,
                         (float*)r, c->st);
-  else if (std::is_same<VT, double>::value && operator_mf_preferred(L.g))
-    operator_mf(L.g, L.op_lin, L.w, (const double*)x, (const double*)b, c->op_scr, (double*)r, c->st);
+  else if (std::is_same<VT, double>::value && L.op)
+    operator_mf(L.g, L.op, L.op_w, (const double*)x, (const double*)b, c->op_scr, (double*)r, c->st);
   else
     apply_operator<VT, VT>(L.g, L.rowptr, L.colidx, Ops<VT>::vv(L), Ops<VT>::vp(L), Ops<VT>::pv(L), x, b, r, c->st);
 }
 
-// J x (b null) or b - J x with the FP64 operator of level L: matrix-free in 3D (op_w: the level's w, or a Newton
-// iterate, whose Oseen operator is then never assembled), the assembled blocks otherwise and on the coarsest level.
+// J x (b null) or b - J x with the FP64 operator of level L: matrix-free in 3D (a Newton iterate's Oseen operator is
+// then never assembled), the assembled blocks otherwise and on the coarsest level.
 void apply64(stg_ctx* c, const LevelBufs& L, const double* x, const double* b, double* y) {
-  if (operator_mf_preferred(L.g) && (&L != &c->lv[0] || L.op_w != L.w))
-    operator_mf(L.g, L.op_w != L.w ? L.op_oseen : L.op_lin, L.op_w, x, b, c->op_scr, y, c->st);
+  if (L.op)
+    operator_mf(L.g, L.op, L.op_w, x, b, c->op_scr, y, c->st);
   else
     apply_operator<double, double>(L.g, L.rowptr, L.colidx, L.vv, L.vp, L.pv, x, b, y, c->st);
 }
@@ -804,8 +811,8 @@ stg_status fgmres(stg_ctx* c, const double* b, double* x, int* iters_out, double
 double neg_residual(stg_ctx* c, const double* X, double* r) {
   LevelBufs& F = c->lv.back();
   // the velocity part of an internal vector is laid out exactly like an internal w
-  if (operator_mf_preferred(F.g)) {
-    F.op_w = X;
+  if (F.op) {
+    set_operator(c, X, false);
   } else {
     const AsmCoef cf{c->nu, c->tau, c->opt.gamma1, c->opt.gamma2, 0};
     assemble_level_w(F.g, c->td, cf, X, F.rowptr, F.asm_tab, F.vconst, F.vv, F.nnzb, c->st);
@@ -1032,9 +1039,9 @@ stg_status stg_setup(const stg_mesh* mesh, int k, double nu, double tau, const d
         }
       }
       L.w = dalloc<double>(c, g.nvel);
-      if (operator_mf_preferred(g)) {
-        L.op_lin = dalloc<char>(c, (long long)residual_coef_bytes(g, 8));
-        L.op_oseen = dalloc<char>(c, (long long)residual_coef_bytes(g, 8));
+      if (l > 0 && operator_mf_preferred(g)) {
+        L.op = dalloc<char>(c, (long long)residual_coef_bytes(g, 8));
+        L.op_w = l == nl - 1 ? dalloc<double>(c, g.nvel) : L.w;
       }
       L.asm_tab = dalloc<double>(c, assemble_table_doubles(g.dim, k));
       L.vconst = dalloc<double>(c, L.nnzb * g.NV * g.NV);
@@ -1055,7 +1062,7 @@ stg_status stg_setup(const stg_mesh* mesh, int k, double nu, double tau, const d
     }
     if (scratch) c->inv_scratch = dalloc<char>(c, (long long)scratch);
     if (scratch2) c->inv_scratch2 = dalloc<char>(c, (long long)scratch2);
-    if (c->lv.back().op_lin) c->op_scr = dalloc<double>(c, residual_scratch(c->lv.back().g));
+    if (c->lv.back().op) c->op_scr = dalloc<double>(c, residual_scratch(c->lv.back().g));
     if (c->lv.back().mf) c->mf_scr = dalloc<float>(c, residual_scratch(c->lv.back().g));
     c->inv_flags = dalloc<int>(c, c->lv.back().g.n_cells);
     if (mesh->n_levels > 2) c->inv_flags2 = dalloc<int>(c, c->lv[mesh->n_levels - 2].g.n_cells);

@@ -70,6 +70,8 @@ void residual_mf(const Geom& g, const void* coef, const float* w, const float* x
 // internal layout); coef: residual_coef_bytes(g, 8) bytes from operator_coef, scratch: residual_scratch(g) doubles.
 bool operator_mf_preferred(const Geom& g);
 void operator_coef(const Geom& g, const TimeData& td, const AsmCoef& cf, void* dst, cudaStream_t st);
+// Newton's term on or off in coef.
+void operator_set_newton(void* coef, bool newton, cudaStream_t st);
 void operator_mf(const Geom& g, const void* coef, const double* w, const double* x, const double* b, double* scratch,
                  double* out, cudaStream_t st);
 

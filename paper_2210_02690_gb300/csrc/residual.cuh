@@ -127,7 +127,7 @@ struct MfCoef {
   T sa[5];        // tau w_a |det|
   T sc[3];        // 2 / h_e
   T nu, g1[3], g2[3];  // viscosity; gamma1 nu / h_e, gamma2 / h_e
-  int newton;
+  int newton;  // not 0: with Newton's term
 };
 
 // Pressure coefficients of a cell and Radau node, and the same padded to whole 16-byte loads of the table.

@@ -1,6 +1,8 @@
 // The FP64 operator without a matrix: J x and b - J x in 3D.
 #include "residual.cuh"
 
+#include <cstddef>
+
 namespace stg {
 
 // GB300's FP64 pipe bounds both forms.  In 3D the assembled one takes ((k+1) d)^2 multiply-adds a node pair (and 16.8 GB
@@ -10,6 +12,10 @@ bool operator_mf_preferred(const Geom& g) { return g.dim == 3; }
 
 void operator_coef(const Geom& g, const TimeData& td, const AsmCoef& cf, void* dst, cudaStream_t st) {
   upload_coefficients<3, 3, double>(g, td, cf, dst, st);
+}
+
+void operator_set_newton(void* coef, bool newton, cudaStream_t st) {
+  STG_CUDA_OK(cudaMemsetAsync((char*)coef + offsetof(MfCoef<double>, newton), newton ? 1 : 0, sizeof(int), st));
 }
 
 void operator_mf(const Geom& g, const void* coef, const double* w, const double* x, const double* b, double* scratch,

@@ -21,6 +21,7 @@
 // joins V_s as well (a second group of nt slots in every vertex plane, identity
 // rows where unused); removed cells' pressures are identity rows.
 #include <algorithm>
+#include <string>
 #include <vector>
 
 #include "coarse.cuh"
@@ -413,6 +414,9 @@ void CoarseSolver<T>::init(const Geom& geom, bool pure_dirichlet) {
   v.mV = (int)(pn * geom.NV + (has_obstacle(geom) ? 2 : 1) * geom.nt);
   v.mI = (int)((long long)(geom.r - 1) * pn * geom.NV + (long long)geom.n[1] * geom.n[2] * geom.NP - geom.nt);
   const long long mV = v.mV, mI = v.mI, nsi = v.nsi, nsv = v.nsv;
+  if (std::max(mI, mV) > gj_max_rows<T>())
+    throw Error{STG_EINVAL, "coarsest level: a cell column of " + std::to_string(std::max(mI, mV)) +
+                                " unknowns; the direct solver takes " + std::to_string(gj_max_rows<T>())};
   auto alloc = [&](T** p, long long n) {
     STG_CUDA_OK(cudaMalloc(p, sizeof(T) * (n > 0 ? n : 1)));
     owned.push_back(*p);

@@ -17,6 +17,11 @@ struct GjScratch {
   int *piv = nullptr, *pos = nullptr, *fail = nullptr;
 };
 inline long long gj_panel_values(long long m_max) { return 3 * 32 * m_max + 32; }
+// 512 threads hold 19 (FP32) or 18 (FP64) rows of a panel each.
+template <typename T>
+constexpr int gj_max_rows() {
+  return sizeof(T) == 4 ? 9728 : 9216;
+}
 // In-place inverses of `batch` m x m row-major matrices by Gauss-Jordan with partial pivoting;
 // status gets 1 + the index of a singular matrix (coarse_gj.cu).
 template <typename T>

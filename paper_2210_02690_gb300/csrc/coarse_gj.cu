@@ -589,6 +589,7 @@ static bool rgj_invert(int, double* const*, int, int*, cudaStream_t) { return fa
 template <typename T>
 void gj_invert(int m, T* const* A, int batch, int* status, const GjScratch<T>& s, cudaStream_t st) {
   if (batch <= 0 || m <= 0) return;
+  if (m > gj_max_rows<T>()) throw Error{STG_EINVAL, "coarse block larger than its inversion takes"};
   if (rgj_invert(m, A, batch, status, st)) return;
   // the panel's R W values of a thread fit 72 registers (512 threads have 128 each); FP64 halves W.  FP32 up to
   // 1024 rows in the operations and order of the forms it replaces (coarse factors of 2D levels keep their bits).
@@ -604,8 +605,8 @@ void gj_invert(int m, T* const* A, int batch, int* status, const GjScratch<T>& s
     invert_by_panels<T, 9, 8 / D, false>(m, A, batch, 0, status, s, st);
   else if (m <= 9216)
     invert_by_panels<T, 18, 4 / D, false>(m, A, batch, 0, status, s, st);
-  else
-    throw Error{STG_EINVAL, "coarse block of more than 9216 unknowns"};
+  else if constexpr (F32)
+    invert_by_panels<T, 19, 4, false>(m, A, batch, 0, status, s, st);
 }
 
 template void gj_invert<float>(int, float* const*, int, int*, const GjScratch<float>&, cudaStream_t);

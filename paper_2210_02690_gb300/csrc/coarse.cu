@@ -432,25 +432,6 @@ void CoarseSolver<T>::init(const Geom& geom, bool pure_dirichlet) {
   alloc(&GL, nsv * mV * mV);
   alloc(&GU, nsv * mV * mV);
   alloc(&bV, nsv * mV);
-  {
-    // scratch of the Gauss-Jordan inverses: a second copy of every block of a batch, its panels, and
-    // the pivot rows
-    const long long nb = std::max(nsi, nsv), mm = std::max(mI, mV);
-    T *alt = nullptr, *pan = nullptr;
-    alloc(&alt, nb * mm * mm);
-    alloc(&pan, nb * gj_panel_values(mm));
-    std::vector<T*> ha(nb), hp(nb);
-    for (long long b = 0; b < nb; ++b) {
-      ha[b] = alt + b * mm * mm;
-      hp[b] = pan + b * gj_panel_values(mm);
-    }
-    gj.alt = upload_ptrs(ha, owned);
-    gj.panel = upload_ptrs(hp, owned);
-    STG_CUDA_OK(cudaMalloc(&gj.piv, sizeof(int) * nb * (2 * mm + 1)));
-    owned.push_back(gj.piv);
-    gj.pos = gj.piv + nb * mm;
-    gj.fail = gj.pos + nb * mm;
-  }
   alloc(&xV, nsv * mV);
   alloc(&bI, nsi * mI);
   alloc(&gI, nsi * mI);
@@ -598,6 +579,34 @@ void CoarseSolver<T>::init(const Geom& geom, bool pure_dirichlet) {
     curL.swap(newL);
     curU.swap(newU);
   }
+  // Scratch of the inversions.  Their second blocks are arrays that are written only after the inversion: W for the
+  // interiors where it is large enough (order 2), GL for the planes (plane 0, the top, has no GL).
+  {
+    const long long nI = gj_by_panels<T>(mI) ? nsi : 0, nV = gj_by_panels<T>(mV) ? std::max<long long>(1, nsv / 2) : 0;
+    const long long nb = std::max(nI, nV), mm = std::max(nI ? mI : 0, nV ? mV : 0);
+    if (nI && mI <= 2 * mV) {
+      d_alt = d_W;
+    } else if (nI) {
+      T* alt = nullptr;
+      alloc(&alt, nsi * mI * mI);
+      std::vector<T*> pa;
+      for (long long s = 0; s < nsi; ++s) pa.push_back(alt + s * mI * mI);
+      d_alt = upload_ptrs(pa, owned);
+    }
+    d_top_alt = upload_ptrs(std::vector<T*>{GL}, owned);
+    if (nb) {
+      T* pan = nullptr;
+      const long long values = std::max(nI ? gj_panel_values<T>(mI) : 0, nV ? gj_panel_values<T>(mV) : 0);
+      alloc(&pan, nb * values);
+      std::vector<T*> pp;
+      for (long long b = 0; b < nb; ++b) pp.push_back(pan + b * values);
+      gj.panel = upload_ptrs(pp, owned);
+      STG_CUDA_OK(cudaMalloc(&gj.piv, sizeof(int) * nb * (2 * mm + 1)));
+      owned.push_back(gj.piv);
+      gj.pos = gj.piv + nb * mm;
+      gj.fail = gj.pos + nb * mm;
+    }
+  }
   std::vector<T*> top{v.D}, topb{bV}, topx{xV};
   d_top = upload_ptrs(top, owned);
   d_topb = upload_ptrs(topb, owned);
@@ -711,7 +720,9 @@ void CoarseSolver<T>::factor(const int* rowptr, const int* colidx, const double*
     STG_LAUNCH_OK();
   }
   // interiors: A_II^{-1}, W = A_II^{-1} A_IV, C = A_VI W, S = A_VV - C (scattered)
-  gj_invert<T>((int)mI, d_AII, (int)nsi, v.status, gj, st);
+  GjScratch<T> scr = gj;
+  scr.alt = d_alt;
+  gj_invert<T>((int)mI, d_AII, (int)nsi, v.status, scr, st);
   const T one = 1, zero = 0, mone = -1;
   gemm2<T>((int)mI, (int)(2 * mV), (int)mI, one, d_AII, d_AIV, nullptr, nullptr, zero, d_W, (int)nsi, st);
   gemm2<T>((int)(2 * mV), (int)(2 * mV), (int)mI, one, d_AVI, d_W, nullptr, nullptr, zero, d_C, (int)nsi, st);
@@ -720,7 +731,8 @@ void CoarseSolver<T>::factor(const int* rowptr, const int* colidx, const double*
   // block cyclic reduction of the vertex-plane system
   const int m = (int)mV;
   for (const auto& lv : levels) {
-    gj_invert<T>(m, lv.oD, lv.n_odd, v.status, gj, st);
+    scr.alt = lv.gC;  // GL of the odd planes, in order
+    gj_invert<T>(m, lv.oD, lv.n_odd, v.status, scr, st);
     // [GL_i | GU_i] = D_i^{-1} [L_i | U_i]
     gemm2<T>(m, m, m, one, lv.gA, lv.gB, nullptr, nullptr, zero, lv.gC, 2 * lv.n_odd, st);
     // PL_j = L_j D_{j-st}^{-1}, PR_j = U_j D_{j+st}^{-1} (the solve's forward products)
@@ -730,7 +742,8 @@ void CoarseSolver<T>::factor(const int* rowptr, const int* colidx, const double*
     // L_j <- -L_j GL_{j-st}, U_j <- -U_j GU_{j+st}, into new blocks
     gemm2<T>(m, m, m, mone, lv.uA, lv.uB, nullptr, nullptr, zero, lv.uC, lv.n_left + lv.n_right, st);
   }
-  gj_invert<T>(m, d_top, 1, v.status, gj, st);
+  scr.alt = d_top_alt;
+  gj_invert<T>(m, d_top, 1, v.status, scr, st);
 }
 
 template <typename T>

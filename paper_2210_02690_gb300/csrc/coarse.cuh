@@ -8,15 +8,24 @@
 
 namespace stg {
 
-// Scratch of gj_invert for batches of matrices of up to m_max rows: device arrays of pointers to one m_max x m_max
-// block and three m_max x 32 panels per matrix (panel values, multipliers, pivot rows; 32 reciprocal pivots behind),
-// and per matrix m_max pivot rows (piv), m_max row positions (pos) and a failure flag.
+// Scratch of gj_invert for the matrices that go by panels (FP32 beyond the 256 rows of the on-chip form, FP64): device
+// arrays of pointers to one m x m block and gj_panel_values(m) values per matrix, and per matrix m pivot rows (piv),
+// m row positions (pos) and a failure flag.
 template <typename T>
 struct GjScratch {
-  T **alt = nullptr, **panel = nullptr;
+  T* const* alt = nullptr;
+  T** panel = nullptr;
   int *piv = nullptr, *pos = nullptr, *fail = nullptr;
 };
-inline long long gj_panel_values(long long m_max) { return 3 * 32 * m_max + 32; }
+template <typename T>
+bool gj_by_panels(long long m) {
+  return sizeof(T) == 8 || m > 256;
+}
+// The panel, and for FP32 up to 511 rows its multipliers, its pivot rows and 32 reciprocal pivots behind them.
+template <typename T>
+long long gj_panel_values(long long m) {
+  return sizeof(T) == 8 ? 16 * m : (m < 512 ? 3 * 32 * m + 32 : 32 * m);
+}
 // 512 threads hold 19 (FP32) or 18 (FP64) rows of a panel each.
 template <typename T>
 constexpr int gj_max_rows() {
@@ -86,6 +95,8 @@ struct CoarseSolver {
   T **d_bI = nullptr, **d_gI = nullptr, **d_xVs = nullptr, **d_xI = nullptr;
   T **d_cA0 = nullptr, **d_cx0 = nullptr, **d_cA1 = nullptr, **d_cx1 = nullptr, **d_cy = nullptr;
   T **d_top = nullptr, **d_topb = nullptr, **d_topx = nullptr;
+  T** d_alt = nullptr;  // the second blocks of the interiors' inversion; the planes take GL's
+  T** d_top_alt = nullptr;
   GjScratch<T> gj;
   std::vector<CrLevel<T>> levels;
   std::vector<void*> owned;

@@ -52,3 +52,27 @@ def test_larger_blocks_are_refused_at_set_up(form, n, k):
     with pytest.raises(StgError) as e:
         Solver(spec, k, NU, TAU, w, vcycle_prec=form, factor_prec=form)
     assert e.value.status == 1 and "coarsest level" in str(e.value)
+
+
+def test_inversion_scratch_is_paid_for_only_where_it_is_used():
+    """FP32 blocks of 253 rows are inverted on chip, blocks of 260 by panels into a second copy that an array of the
+    factorisation lends (W); neither size allocates a copy of its blocks.  The memory per unknown of order 2's arrays,
+    counted from their sizes, is the bound."""
+    from paper_2210_02690_gb300 import Solver
+    for ny in (36, 37):
+        nx, nsv = 512, 513
+        spec = si.MeshSpec(2, (nx, ny), (0.0, 0.0), (float(nx) / ny, 1.0), 1, FACES)
+        mI, mV = 7 * ny + 1, 4 * ny + 3
+        # A_II, A_IV, A_VI, W, C; D, L, U, GL, GU; per level PL, PR and new L, U of every even plane
+        levels = sum(4 * len(range(0, nsv, 2 * s)) for s in (2 ** i for i in range(10)))
+        arrays = 4 * (nx * (mI * mI + 6 * mI * mV + 4 * mV * mV) + (5 * nsv + levels) * mV * mV)
+        w = torch.from_numpy(np.ascontiguousarray(si.fourier_w(spec, 0)).ravel()).cuda()
+        used = []
+        for form in ("f32", "f64"):
+            torch.cuda.synchronize()
+            free = torch.cuda.mem_get_info()[0]
+            s = Solver(spec, 0, NU, TAU, w, vcycle_prec="f32", factor_prec="f32", coarse_prec=form, gmres_restart=1)
+            used.append(free - torch.cuda.mem_get_info()[0])
+            s.close()
+        # the two forms differ by 4 bytes a value of the arrays, and by the panels (2% here)
+        assert used[1] - used[0] <= 1.06 * arrays

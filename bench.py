@@ -292,7 +292,7 @@ FP64_NOMINAL_TFLOPS = 1.25  # GB300 dense FP64, nominal
 
 def colour_fraction(k: int, form: str, ms: float, launches: int, patches: int, peak: float,
                     variant: int | None = None) -> dict:
-    """HBM fraction of the finest level's colour kernels (2D): algorithmic bytes (every J_K^{-1}
+    """HBM fraction of the finest level's patch kernel (2D): algorithmic bytes (every J_K^{-1}
     in the form's factor precision, r gathered, y stored) over their CUDA-event time."""
     n = 21 * (k + 1)
     fs = {"f64": 8, "f32": 4, "bf16": 2}[form]
@@ -395,7 +395,6 @@ def gpu_arm(args) -> None:
             tuned = solver.autotune()
         timed_steps(solver, w, b, x, args.warmup, torch)
         steps = args.steps if name == "f32" else max(3, args.steps // 2)
-        solver.profile(True)
         if name == "f32":
             launches0 = solver.kernel_launches()
         barrier(world)
@@ -425,6 +424,9 @@ def gpu_arm(args) -> None:
                             "variants": ",".join(str(v) for v in solver.colour_variants())},
                "time_to_tol_ms": e[1].elapsed_time(e[2]), "rel_res": rel_s, "clocks": clocks,
                "value": aggregate_rate(per_cycle * its, steps, world, ms_max)}
+        # the patch kernel, in steps of its own: the events are not part of the timed ones
+        solver.profile(True, as_launched=True)
+        timed_steps(solver, w, b, x, min(steps, 5), torch)
         pms, plaunch, ppatch = solver.profile_read()
         res["colour_kernel"] = (pms, plaunch, ppatch)
         solver.profile(False)
@@ -465,7 +467,7 @@ def gpu_arm(args) -> None:
     r32 = results["f32"]
     pms, plaunch, ppatch = r32["colour_kernel"]
     npatch = 21 * (k + 1)
-    # algorithmic bytes of one colour-kernel launch: each patch streams its J_K^{-1}
+    # algorithmic bytes of one patch-kernel launch (all patches): each patch streams its J_K^{-1}
     # (npatch^2 FP32 values), gathers npatch residual values and stores npatch values of y
     bytes_per_patch = npatch * npatch * 4 + 2 * npatch * 4
     avg_ms = pms / max(plaunch, 1)

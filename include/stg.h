@@ -245,7 +245,9 @@ stg_status stg_get_local_inverse(const stg_ctx* ctx, int level, long long cell, 
  * sweep per V-cycle (the last post-smoothing sweep, or the last pre-smoothing
  * sweep when nu2 = 0; the last sweep of stg_smooth), which is launched colour
  * by colour for that (other sweeps take all patches in one launch), and
- * accumulates their device time; stg_profile(ctx, 0) stops and resets.  The
+ * accumulates their device time.  stg_profile(ctx, 2) records them around the
+ * launch as every other sweep makes it: one per sampled sweep of the averaged
+ * smoother, 2^d of the coloured one.  stg_profile(ctx, 0) stops and resets.  The
  * V-cycle graph is recaptured when the setting changes.  stg_profile_read
  * returns the accumulated milliseconds, the number of launches and the number
  * of patches they processed (host pointers, each may be NULL). */

@@ -377,9 +377,10 @@ class Solver:
                                                                   out.ctypes.data_as(ctypes.c_void_p)))
         return out
 
-    def profile(self, enable: bool):
-        """Start (and reset) or stop CUDA-event timing of the finest-level colour kernels."""
-        self._call(self.lib.stg_profile, 1 if enable else 0)
+    def profile(self, enable: bool, as_launched: bool = False):
+        """Start (and reset) or stop CUDA-event timing of the finest-level patch kernels, colour by colour or
+        as an ordinary sweep launches them."""
+        self._call(self.lib.stg_profile, (2 if as_launched else 1) if enable else 0)
 
     def profile_read(self):
         """(device milliseconds, launches, patches) accumulated since profiling started."""

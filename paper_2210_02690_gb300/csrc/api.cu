@@ -238,7 +238,7 @@ struct stg_ctx {
   int graph_prof_events = 0;
   long long graph_prof_patches = 0;
   // instrumentation: CUDA events around the finest-level colour kernels
-  bool prof_on = false;
+  int prof_on = 0;  // 1: the sampled sweep colour by colour, 2: as every other sweep is launched
   std::vector<cudaEvent_t> prof_ev;
   int prof_used = 0;
   double prof_ms = 0.0;
@@ -464,7 +464,7 @@ void smooth_level(stg_ctx* c, int l, int sweeps, bool x_zero) {
   const FT* jinv = (const FT*)L.jinv;
   const int ncol = 1 << g.dim;
   for (int s = 0; s < sweeps; ++s) {
-    // with profiling on, the colour launches of one sweep per V-cycle are bracketed by events
+    // with profiling on, the patch launches of one sweep per V-cycle are bracketed by events
     // (the last post-smoothing sweep of the finest level; the last pre-smoothing sweep when
     // there is no post-smoothing): each event node is a graph node of its own, so a sample
     // keeps the timed cycle close to the uninstrumented one
@@ -475,10 +475,11 @@ void smooth_level(stg_ctx* c, int l, int sweeps, bool x_zero) {
         residual<VT>(c, L, x, b, r);
         res = r;
       }
-      // one launch over all patches; a profiled sweep takes them colour by colour
+      // one launch over all patches; a sampled sweep may take them colour by colour
       if (prof_sweep && c->prof_on && l == (int)c->lv.size() - 1) {
-        for (int col = 0; col < ncol; ++col) {
-          const long long p0 = g.coff[col], cnt = g.coff[col + 1] - p0;
+        const int parts = c->prof_on == 1 ? ncol : 1;
+        for (int part = 0; part < parts; ++part) {
+          const long long p0 = parts == 1 ? 0 : g.coff[part], cnt = (parts == 1 ? g.n_cells : g.coff[part + 1]) - p0;
           const bool prof = c->prof_used + 2 <= (int)c->prof_ev.size();
           if (prof) record_event(c->prof_ev[c->prof_used], c->st);
           vanka_patches<VT, FT>(g, p0, cnt, jinv, res, y, c->st, L.colour_variant);
@@ -1492,20 +1493,21 @@ stg_status stg_get_local_inverse(const stg_ctx* cc, int level, long long cell, d
 
 stg_status stg_profile(stg_ctx* c, int enable) {
   if (!c) return STG_EINVAL;
+  const int mode = enable == 0 || enable == 2 ? enable : 1;
   try {
-    if (enable && c->prof_ev.empty()) {
+    if (mode && c->prof_ev.empty()) {
       const int per_cycle = 2 * (1 << c->mesh.dim);  // one sweep's colour launches per V-cycle
       c->prof_ev.resize(per_cycle);
       for (auto& e : c->prof_ev) STG_CUDA_OK(cudaEventCreate(&e));
     }
-    if ((bool)enable != c->prof_on) {
+    if (mode != c->prof_on) {
       STG_CUDA_OK(cudaStreamSynchronize(c->st));
       if (c->graph) {  // the captured V-cycle changes with the instrumentation
         STG_CUDA_OK(cudaGraphExecDestroy(c->graph));
         c->graph = nullptr;
       }
     }
-    c->prof_on = enable != 0;
+    c->prof_on = mode;
     c->prof_used = 0;
     c->prof_pending_patches = 0;
     c->prof_ms = 0.0;

@@ -870,13 +870,16 @@ double tune_level(stg_ctx* c, int l, int reps) {
   STG_CUDA_OK(cudaEventCreate(&e1));
   double best = 1e30;
   int bestv = L.colour_variant;
-  // a sweep's patches as the smoother launches them: all at once, or colour by colour (coloured mode)
-  const int parts = c->opt.smoother == STG_VANKA_AVERAGED ? 1 : 1 << L.g.dim;
+  // a sweep's patches as the smoother launches them: all at once, or colour by colour, added into a vector (coloured
+  // mode, which does not use y otherwise; it is at least as long as a vector)
+  const bool averaged = c->opt.smoother == STG_VANKA_AVERAGED;
+  if (!averaged) fill_zero<VT>(L.g.N, (VT*)L.y, c->st);
   auto sweep = [&](int v) {
-    for (int i = 0; i < parts; ++i) {
-      const long long p0 = parts == 1 ? 0 : L.g.coff[i], p1 = parts == 1 ? L.g.n_cells : L.g.coff[i + 1];
-      vanka_patches<VT, FT>(L.g, p0, p1 - p0, (const FT*)L.jinv, (const VT*)L.r, (VT*)L.y, c->st, v);
-    }
+    if (averaged)
+      vanka_patches<VT, FT>(L.g, 0, L.g.n_cells, (const FT*)L.jinv, (const VT*)L.r, (VT*)L.y, c->st, v);
+    else
+      for (int i = 0; i < 1 << L.g.dim; ++i)
+        vanka_colour<VT, FT>(L.g, i, (const FT*)L.jinv, (const VT*)L.r, (VT*)L.y, (VT)1, c->st, v);
   };
   for (int v = 0; v < kColourVariants; ++v) {
     for (int w = 0; w < 2; ++w) sweep(v);  // warm-up
@@ -1051,7 +1054,9 @@ stg_status stg_setup(const stg_mesh* mesh, int k, double nu, double tau, const d
       L.r = dalloc<char>(c, (long long)vts * g.N);
       STG_CUDA_OK(cudaMemset(L.x, 0, vts * g.N));
       if (l > 0) {
-        L.colour_variant = default_colour_variant(g, opt->factor_prec);
+        // the averaged smoother takes all patches in one launch, the coloured one a colour
+        const int launches = opt->smoother == STG_VANKA_COLOURED ? 1 << g.dim : 1;
+        L.colour_variant = default_colour_variant(g, opt->factor_prec, (g.n_cells + launches - 1) / launches);
         L.y = dalloc<char>(c, (long long)vts * g.n_cells * g.npatch);
         L.jinv = dalloc<char>(c, (long long)fsize(opt->factor_prec) * patch_stride(g.npatch) * g.n_cells);
         const int cf32 = opt->factor_prec != STG_F64 ? 1 : 0;

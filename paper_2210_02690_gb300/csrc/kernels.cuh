@@ -101,8 +101,8 @@ bool invert_panels(const Geom& g, const int* rowptr, const double* vv, const dou
 constexpr int kColourWarpVariants = 9;
 constexpr int kColourVariants = 17;
 constexpr int kColourWarpDefault = 4;  // 8 columns, 256 threads
-// The variant a level starts with; the autotuner may replace it.
-int default_colour_variant(const Geom& g, int factor_prec);
+// The variant a level starts with, for launches of this many patches; the autotuner may replace it.
+int default_colour_variant(const Geom& g, int factor_prec, long long patches);
 template <typename VT, typename FT>
 void vanka_patches(const Geom& g, long long p0, long long cnt, const FT* jinv, const VT* r, VT* y, cudaStream_t st,
                    int variant);

@@ -1469,15 +1469,23 @@ void run_patches(const Geom& g, long long p0, long long cnt, const FT* jinv, con
 }  // namespace
 
 // Two stages keep the most CTAs on an SM, and bytes in flight are what the staged form needs; the factor may be
-// large before one or two CTAs are left (44 KB at n = 105 in FP32).  Beyond, and in FP64 from n = 60 on (bound by the
-// FP64 pipe), one warp per patch.  Whole sweeps (residual and update included) on 65536 patches, 4 stages
-// -> this choice: FP32 n = 63 299 -> 280 us, 84 464 -> 450, 105 814 -> 652 (one warp per patch 687); BF16, whose
-// issue-bound product wants two rows a thread, n = 42 (90112) 202 -> 173, 84 387 -> 330, 105 572 -> 461; FP64 n = 63
-// 1886 -> 966.  3D n = 85, 32768 patches: FP32 349 -> 213.  FP32 n = 120, 170: two stages 301, 329, one warp 284, 323.
-int default_colour_variant(const Geom& g, int factor_prec) {
+// large before one or two CTAs are left (44 KB at n = 105 in FP32).  Beyond, and for large launches in FP64 from n = 60
+// on (bound by the FP64 pipe), one warp per patch.  Whole sweeps (residual and update included) on 65536 patches in one
+// launch, 4 stages -> this choice: FP32 n = 63 299 -> 280 us, 84 464 -> 450, 105 814 -> 652 (one warp per patch 687);
+// BF16, whose issue-bound product wants two rows a thread, n = 42 (90112) 202 -> 173, 84 387 -> 330, 105 572 -> 461;
+// FP64 n = 63 1886 -> 966.  3D n = 85, 32768 patches: FP32 349 -> 213.  FP32 n = 120, 170: two stages 301, 329, one warp
+// 284, 323.
+// A launch of few patches (small levels; the coloured smoother takes 2^d launches a sweep) is a chain of latencies: a warp's
+// loads against one bulk copy, and 2 rows a thread leave half the warps.  FP64 sweeps, one warp per patch -> two stages:
+// coloured, 64 patches a launch n = 60 142 -> 121 us, 63 111 -> 90, 84 196 -> 102, 105 177 -> 112; 1024 n = 63 232 -> 200,
+// 84 505 -> 291, 105 468 -> 460; 4096 n = 63 503 -> 505, 105 1173 -> 1300; averaged, 1024 n = 84 93 -> 60, 4096 133 -> 133
+// (n = 63 84 -> 85, 105 200 -> 230): the line is at 2048.  BF16, two rows -> one: coloured, 64 n = 42 78 -> 70, 84 86 -> 83; 256
+// n = 42 71 -> 68; 1024 77 -> 78: at 512.
+int default_colour_variant(const Geom& g, int factor_prec, long long patches) {
   const int n = g.npatch, size = factor_prec == STG_F64 ? 8 : (factor_prec == STG_F32 ? 4 : 2);
-  if (factor_prec == STG_F64 ? n < 60 : n * n * size <= 48 * 1024) return factor_prec == STG_BF16 ? 15 : 11;
-  return 3;
+  if (factor_prec == STG_F64) return n < 60 || (patches <= 2048 && n * n * size <= 96 * 1024) ? 11 : 3;
+  if (n * n * size > 48 * 1024) return 3;
+  return factor_prec == STG_BF16 && patches > 512 ? 15 : 11;
 }
 
 template <typename VT, typename FT>

@@ -385,8 +385,7 @@ bool invert_panels(const Geom& g, const int* rowptr, const double* vv, const dou
     case 180:  // order 4, k = 2
       launch<6, 23, 1, 1, FT>(g, rowptr, vv, vp, pv, jinv, stride, flags, st);
       return true;
-    case 255:  // 3D k = 2: more registers than one CTA has
-      if (g.dim != 3) return false;  // the cluster form has no removed-cell path
+    case 255:  // 3D k = 2: more registers than one CTA has (no 2D patch has this size, so no removed cells)
       launch<8, 16, 2, 1, FT>(g, rowptr, vv, vp, pv, jinv, stride, flags, st);
       return true;
     default: return false;

@@ -34,8 +34,8 @@ void residual_mf(const Geom& g, const void* coef, const float* w, const float* x
       case 2: return run3d<2, float>(g, coef, w, x, b, scratch, out, st);
       default: return run3d<3, float>(g, coef, w, x, b, scratch, out, st);
     }
-  if (g.nt == 2) return run2d<5, 2, float>(g, coef, w, x, b, out, st);
-  run2d<5, 3, float>(g, coef, w, x, b, out, st);
+  if (g.nt == 2) return run2d<2, float>(g, coef, w, x, b, out, st);
+  run2d<3, float>(g, coef, w, x, b, out, st);
 }
 
 }  // namespace stg

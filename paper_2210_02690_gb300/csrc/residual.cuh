@@ -423,7 +423,7 @@ __device__ __forceinline__ void cell_operator(const MfCoef<T>& cf, int a, int c,
   }
 }
 
-// Dirichlet faces of a cell (bit 2 e + side), the obstacle's included.
+// Dirichlet faces of a cell (bit 2 e + side).
 template <int DIM>
 __device__ __forceinline__ unsigned cell_faces(const Geom& g, int cx, int cy, int cz) {
   unsigned f = 0;
@@ -433,25 +433,22 @@ __device__ __forceinline__ unsigned cell_faces(const Geom& g, int cx, int cy, in
     if (cc[e] == 0) f |= g.dirichlet & (1u << (2 * e));
     if (cc[e] == g.n[e] - 1) f |= g.dirichlet & (1u << (2 * e + 1));
   }
-  if (DIM == 2 && has_obstacle(g))
-    for (int q = 0; q < 4; ++q)
-      if (face_on_obstacle(g, cx, cy, q >> 1, q & 1)) f |= 1u << q;
   return f;
 }
 
-// 2D: one launch.  A CTA owns 31 cell columns by ty cell rows and walks up the rows; warp v = (a, c), lane =
+// 2D, order 4 (which has no obstacle): one launch.  A CTA owns 31 cell columns by ty cell rows and walks up the rows; warp v = (a, c), lane =
 // cell column, lane 0 the column left of the owned ones.  A node's sum over its cells is formed in
 // registers: the right edge of the left neighbour comes by a shuffle, the top edge of the row below is
 // kept from the previous step (the row below the owned ones is computed for that alone).  Bound by FP32
 // issue; the repeated column and row cost 32/31 and (ty + 1)/ty.
-template <int M, int NT, typename T>
+template <int NT, typename T>
 __global__ void __launch_bounds__(64 * NT, NT == 2 ? 3 : 2) mf_residual2d(Geom g, const MfCoef<T>* __restrict__ cfp,
                                                         const T* __restrict__ table, const T* __restrict__ w,
                                                         const T* __restrict__ x, const T* __restrict__ b,
                                                         T* __restrict__ out, int ty) {
   pdl_wait();
   const MfCoef<T>& cf = *cfp;
-  constexpr int N = M * M, R = M - 1, NV = 2 * NT, NP = kNP<M>;
+  constexpr int M = 5, N = M * M, R = M - 1, NV = 2 * NT, NP = kNP<M>;
   extern __shared__ __align__(16) unsigned char mf_smem[];
   T* sv = reinterpret_cast<T*>(mf_smem);
   T* sw = sv + NV * N * 32;
@@ -461,15 +458,13 @@ __global__ void __launch_bounds__(64 * NT, NT == 2 ? 3 : 2) mf_residual2d(Geom g
   const int y1 = min(y0 + ty, g.n[1]);
   const bool col = cx >= 0 && cx < g.n[0], owned = col && lane > 0;
   const bool last_col = cx == g.n[0] - 1;
-  const bool obst = has_obstacle(g);
   T carry[M];
 #pragma unroll
   for (int i = 0; i < M; ++i) carry[i] = (T)0;
   for (int cy = y0 > 0 ? y0 - 1 : 0; cy < y1; ++cy) {
-    const bool dead = !col || (obst && cell_masked(g, cx, cy));
     T V[N], W[N], P[NP], pp[NP];
     const long long n0 = ((long long)R * cy * g.nn[0] + R * cx) * NV + v;
-    if (dead) {
+    if (!col) {
 #pragma unroll
       for (int i = 0; i < N; ++i) V[i] = W[i] = (T)0;
 #pragma unroll
@@ -485,13 +480,13 @@ __global__ void __launch_bounds__(64 * NT, NT == 2 ? 3 : 2) mf_residual2d(Geom g
 #pragma unroll
       for (int m = 0; m < NP; ++m) P[m] = pc[m];
     }
-    const unsigned faces = dead ? 0u : cell_faces<2>(g, cx, cy, 0);
+    const unsigned faces = col ? cell_faces<2>(g, cx, cy, 0) : 0u;
     const T* rows_c = table + ((a * 16 + faces) * 2 + c) * (N * kNPP<M>);
     pressure_rows<M, N, T>(rows_c, V, pp);
     __syncthreads();  // the cell row below has been read from shared memory
 #pragma unroll
     for (int m = 0; m < NP; ++m) sp[(v * NP + m) * 32 + lane] = pp[m];
-    cell_operator<2, M, NT, T>(cf, a, c, faces, V, W, sv, sw, lane, !dead, [&](int i, int b_) {
+    cell_operator<2, M, NT, T>(cf, a, c, faces, V, W, sv, sw, lane, col, [&](int i, int b_) {
       return x[n0 + ((long long)(i / M) * g.nn[0] + i % M) * NV + 2 * (b_ - a)];
     });
     add_pressure<M, N, T>(rows_c, P, V);
@@ -499,7 +494,7 @@ __global__ void __launch_bounds__(64 * NT, NT == 2 ? 3 : 2) mf_residual2d(Geom g
     if (write && owned) {
       const long long o0 = g.nvel + ((long long)cy * g.n[0] + cx) * (NT * NP) + a * NP;
       for (int m = c; m < NP; m += 2) {
-        const T s = dead ? x[o0 + m] : sp[(2 * a * NP + m) * 32 + lane] + sp[((2 * a + 1) * NP + m) * 32 + lane];
+        const T s = sp[(2 * a * NP + m) * 32 + lane] + sp[((2 * a + 1) * NP + m) * 32 + lane];
         out[o0 + m] = b ? b[o0 + m] - s : s;
       }
     }
@@ -518,9 +513,7 @@ __global__ void __launch_bounds__(64 * NT, NT == 2 ? 3 : 2) mf_residual2d(Geom g
         for (int ix = 0; ix < M; ++ix) {
           if (ix == R && !last_col) break;
           const long long o = ((long long)(R * cy + iy) * g.nn[0] + R * cx + ix) * NV + v;
-          T s = e[ix];
-          if (obst && node_dead(g, R * cx + ix, R * cy + iy)) s = x[o];
-          out[o] = b ? b[o] - s : s;
+          out[o] = b ? b[o] - e[ix] : e[ix];
         }
       }
     }
@@ -530,7 +523,8 @@ __global__ void __launch_bounds__(64 * NT, NT == 2 ? 3 : 2) mf_residual2d(Geom g
 }
 
 // 3D: the cells' contributions E[(v, node)][cell] and the pressure rows, one thread per (cell, component);
-// then mf_nodes3d sums each node's cells.  E (4 * 27 bytes per cell and component) mostly stays in L2.
+// then mf_nodes3d sums each node's cells.  E takes 27 sizeof(T) bytes per cell and component: at 48^3, k = 1 72 MB in
+// FP32, which mostly stays in L2, and 143 MB in FP64, which does not.
 template <int NT, typename T>
 __global__ void __launch_bounds__(96 * NT) mf_cells3d(Geom g, const MfCoef<T>* __restrict__ cfp,
                                                      const T* __restrict__ table, const T* __restrict__ w,
@@ -643,15 +637,15 @@ const T* table_of(const void* coef) {
   return reinterpret_cast<const T*>(static_cast<const char*>(coef) + kTableOffset);
 }
 
-template <int M, int NT, typename T>
+template <int NT, typename T>
 void run2d(const Geom& g, const void* coef, const T* w, const T* x, const T* b, T* out, cudaStream_t st) {
   constexpr int NV = 2 * NT;
-  constexpr size_t smem = sizeof(T) * 32 * NV * (2 * M * M + kNP<M>);
+  constexpr size_t smem = sizeof(T) * 32 * NV * (2 * 25 + kNP<5>);
   if (smem > 48 * 1024)
-    STG_CUDA_OK(cudaFuncSetAttribute(mf_residual2d<M, NT, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    STG_CUDA_OK(cudaFuncSetAttribute(mf_residual2d<NT, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const int nbx = (g.n[0] + 30) / 31;
   const int ty = std::max(1, std::min(16, (int)((long long)nbx * g.n[1] / kMinCtas)));
-  launch_k(mf_residual2d<M, NT, T>, dim3(nbx, (g.n[1] + ty - 1) / ty), dim3(32, NV), smem, st, g, (const MfCoef<T>*)coef,
+  launch_k(mf_residual2d<NT, T>, dim3(nbx, (g.n[1] + ty - 1) / ty), dim3(32, NV), smem, st, g, (const MfCoef<T>*)coef,
            table_of<T>(coef), w, x, b, out, ty);
 }
 

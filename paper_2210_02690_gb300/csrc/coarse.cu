@@ -7,11 +7,12 @@
 //     pressure of the cells of cell column s).  I_s couples only to V_s and
 //     V_{s+1}, so J_0 = [[A_VV, A_VI], [A_IV, A_II]] with block-diagonal A_II;
 //   * the interiors are eliminated in parallel (dense Gauss-Jordan inverses with
-//     partial pivoting, one CTA per slab): S = A_VV - A_VI A_II^{-1} A_IV is block
-//     tridiagonal over the vertex planes;
+//     partial pivoting, on chip or by panels: coarse_gj.cu): S = A_VV - A_VI A_II^{-1}
+//     A_IV is block tridiagonal over the vertex planes;
 //   * S is factored by block cyclic reduction (log2 of the plane count levels,
 //     each a batch of independent dense inverses and products).
-// Everything is FP64.  With Dirichlet data on the whole boundary J_0 has one
+// The operator comes in and the vectors come and go in FP64; the factors and the solve's
+// arithmetic are FP64 or FP32 (T), the caller refines.  With Dirichlet data on the whole boundary J_0 has one
 // constant-pressure null vector per Radau node; the pressure coefficient 0 of
 // cell 0 is then fixed to zero at every Radau node (its row and column become
 // identity rows), which yields the solution with that value for consistent b.

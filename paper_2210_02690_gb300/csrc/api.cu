@@ -190,8 +190,11 @@ struct LevelBufs {
   float *vv32 = nullptr, *vp32 = nullptr, *pv32 = nullptr;
   double* vconst = nullptr;  // the w = 0 assembly (time coupling, viscous, Nitsche), built once
   float *mk32 = nullptr, *ak32 = nullptr;  // Kronecker-split FP32 velocity rows (F32 form, levels >= 1, 2D)
-  void* op = nullptr;      // coefficients of the matrix-free FP64 operator (3D, levels >= 1)
-  double* op_w = nullptr;  // and its velocity: w, on the finest level a copy of w or of a Newton iterate's (then Oseen)
+  // the matrix-free FP64 operator (3D, levels >= 1): coefficients and velocity (w; on the finest level a copy of w or of a
+  // Newton iterate's, then Oseen).  op_mf: it is the level's operator; otherwise (finest level) only a Newton iterate's
+  void* op = nullptr;
+  double* op_w = nullptr;
+  bool op_mf = false;
   float* vd32 = nullptr;  // diagonals of the FP32 velocity blocks (F32 form, levels >= 1, 3D and order 4, k = 0, Oseen)
   float* w32 = nullptr;  // w and coefficients of the matrix-free FP32 residual (F32 form, levels >= 1, 3D and order 4)
   void* mf = nullptr;
@@ -229,6 +232,7 @@ struct stg_ctx {
   int* inv_flags2 = nullptr;
   float* mf_scr = nullptr;     // scratch of the matrix-free residual
   double* op_scr = nullptr;    // and of the matrix-free FP64 operator
+  bool op_iterate = false;     // the finest FP64 operator is a Newton iterate's and the assembled blocks are not
   // FGMRES (finest level, internal layout, FP64)
   double *V = nullptr, *Z = nullptr, *wv = nullptr, *rv = nullptr, *partial = nullptr, *hd = nullptr;
   double *tmp_a = nullptr, *tmp_b = nullptr;
@@ -323,6 +327,7 @@ void set_operator(stg_ctx* c, const double* X, bool newton) {
   LevelBufs& F = c->lv.back();
   STG_CUDA_OK(cudaMemcpyAsync(F.op_w, X, sizeof(double) * F.g.nvel, cudaMemcpyDeviceToDevice, c->st));
   operator_set_newton(F.op, newton, c->st);
+  c->op_iterate = false;
 }
 
 // Assemble every level for the finest-level linearisation velocity in F.w (internal
@@ -426,6 +431,14 @@ void record_event(cudaEvent_t ev, cudaStream_t st) {
     STG_CUDA_OK(cudaEventRecord(ev, st));
 }
 
+// J x (b null) or b - J x with the FP64 operator of level L.
+void apply64(stg_ctx* c, const LevelBufs& L, const double* x, const double* b, double* y) {
+  if (L.op_mf || (c->op_iterate && &L == &c->lv.back()))
+    operator_mf(L.g, L.op, L.op_w, x, b, c->op_scr, y, c->st);
+  else
+    apply_operator<double, double>(L.g, L.rowptr, L.colidx, L.vv, L.vp, L.pv, x, b, y, c->st);
+}
+
 template <typename VT>
 void residual(stg_ctx* c, const LevelBufs& L, const VT* x, const VT* b, VT* r) {
   if (std::is_same<VT, float>::value && L.mf)
@@ -436,19 +449,10 @@ void residual(stg_ctx* c, const LevelBufs& L, const VT* x, const VT* b, VT* r) {
   else if (std::is_same<VT, float>::value && L.mk32)
     apply_operator_kron(L.g, c->td, L.mk32, L.ak32, L.vp32, L.pv32, (const float*)x, (const float*)b,
                         (float*)r, c->st);
-  else if (std::is_same<VT, double>::value && L.op)
-    operator_mf(L.g, L.op, L.op_w, (const double*)x, (const double*)b, c->op_scr, (double*)r, c->st);
+  else if constexpr (std::is_same<VT, double>::value)
+    apply64(c, L, x, b, r);
   else
     apply_operator<VT, VT>(L.g, L.rowptr, L.colidx, Ops<VT>::vv(L), Ops<VT>::vp(L), Ops<VT>::pv(L), x, b, r, c->st);
-}
-
-// J x (b null) or b - J x with the FP64 operator of level L: matrix-free in 3D (a Newton iterate's Oseen operator is
-// then never assembled), the assembled blocks otherwise and on the coarsest level.
-void apply64(stg_ctx* c, const LevelBufs& L, const double* x, const double* b, double* y) {
-  if (L.op)
-    operator_mf(L.g, L.op, L.op_w, x, b, c->op_scr, y, c->st);
-  else
-    apply_operator<double, double>(L.g, L.rowptr, L.colidx, L.vv, L.vp, L.pv, x, b, y, c->st);
 }
 
 // x_zero: the sweeps start from x = 0; x need not hold it (the first update writes every value), except
@@ -609,7 +613,8 @@ void vcycle_body(stg_ctx* c) {
 // One V-cycle; with profiling on, the events of the colour kernels are read
 // back after the cycle (the caller synchronises before the next one).
 void run_vcycle(stg_ctx* c) {
-  if (c->opt.use_graph) {
+  // (captured with the assembled operator; a Newton iterate's is applied without a graph)
+  if (c->opt.use_graph && !(c->op_iterate && vc64(c))) {
     if (!c->graph) {
       cudaGraph_t graph = nullptr;
       const long long before = launch_counter();
@@ -812,8 +817,9 @@ stg_status fgmres(stg_ctx* c, const double* b, double* x, int* iters_out, double
 double neg_residual(stg_ctx* c, const double* X, double* r) {
   LevelBufs& F = c->lv.back();
   // the velocity part of an internal vector is laid out exactly like an internal w
-  if (F.op) {
+  if (F.op) {  // nothing to assemble for a Newton iterate
     set_operator(c, X, false);
+    c->op_iterate = !F.op_mf;
   } else {
     const AsmCoef cf{c->nu, c->tau, c->opt.gamma1, c->opt.gamma2, 0};
     assemble_level_w(F.g, c->td, cf, X, F.rowptr, F.asm_tab, F.vconst, F.vv, F.nnzb, c->st);
@@ -1043,7 +1049,8 @@ stg_status stg_setup(const stg_mesh* mesh, int k, double nu, double tau, const d
         }
       }
       L.w = dalloc<double>(c, g.nvel);
-      if (l > 0 && operator_mf_preferred(g)) {
+      L.op_mf = l > 0 && operator_mf_preferred(g, opt->linearisation == STG_NEWTON);
+      if (L.op_mf || (l > 0 && l == nl - 1 && g.dim == 3)) {
         L.op = dalloc<char>(c, (long long)residual_coef_bytes(g, 8));
         L.op_w = l == nl - 1 ? dalloc<double>(c, g.nvel) : L.w;
       }

@@ -68,7 +68,7 @@ void residual_mf(const Geom& g, const void* coef, const float* w, const float* x
 
 // The FP64 operator without a matrix (3D, residual64.cu): out = b - J x, or J x (b null), at linearisation velocity w (FP64,
 // internal layout); coef: residual_coef_bytes(g, 8) bytes from operator_coef, scratch: residual_scratch(g) doubles.
-bool operator_mf_preferred(const Geom& g);
+bool operator_mf_preferred(const Geom& g, bool newton);
 void operator_coef(const Geom& g, const TimeData& td, const AsmCoef& cf, void* dst, cudaStream_t st);
 // Newton's term on or off in coef.
 void operator_set_newton(void* coef, bool newton, cudaStream_t st);

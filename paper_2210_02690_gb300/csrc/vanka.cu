@@ -39,7 +39,7 @@ __device__ __forceinline__ void op_pres_row(const Geom& g, const MT* __restrict_
 // Whole steps: 256^2 k = 3 42.1 -> 40.1 ms, 256^2 k = 2 21.9 -> 20.4, 704x128 FP64 form 70.3 -> 67.9,
 // 8x8 k = 0 3.41 -> 3.02 (latency), same bits.
 // DIAG (one Radau node, Oseen, no obstacle): the components do not couple either, and vv holds the DIM diagonal values
-// of a block alone.
+// of a block alone (48^3 k = 0 FP32: whole sweep 1218 -> 950 us against the full blocks).
 template <int DIM, int NT, typename MT, typename VT, bool DIAG = false>
 __global__ void __launch_bounds__(256) op_rows(Geom g, const int* __restrict__ rowptr, const int* __restrict__ colidx,
                                                const MT* __restrict__ vv, const MT* __restrict__ vp,
@@ -846,12 +846,15 @@ __device__ __forceinline__ void patch_bases(const Geom& g, long long p, int& col
 }
 
 // y_K = J_K^{-1} R_K r for the patches p0 .. p0 + cnt - 1, one warp per patch, loads straight from global
-// memory.  STORE: out[p n + row] = y (out: one block of n values per patch); otherwise out[dof] += scale y
+// memory.  Without STORE the launches are small (one colour), so registers go to loads in flight and not to warps:
+// left to itself the compiler keeps 60 registers and hardly a load (coloured sweeps, 64 patches a launch: FP64 n = 170
+// 2854 -> 1339 us, FP32 n = 170 400 -> 300, n = 120 188 -> 139).  STORE: out[p n + row] = y (out: one block of n values per patch); otherwise out[dof] += scale y
 // (the patches of the range share no DoF).
 template <typename VT, typename FT, int RPL, int CB, bool STORE>
-__global__ void __launch_bounds__(512) vanka_colour_kernel(Geom g, long long p0, long long cnt,
-                                                           const FT* __restrict__ jinv, long long stride,
-                                                           const VT* __restrict__ r, VT* __restrict__ out, VT scale) {
+__global__ void __launch_bounds__(512, STORE ? 0 : 1) vanka_colour_kernel(Geom g, long long p0, long long cnt,
+                                                                          const FT* __restrict__ jinv, long long stride,
+                                                                          const VT* __restrict__ r, VT* __restrict__ out,
+                                                                          VT scale) {
   pdl_wait();
   using AT = typename AccT<VT>::type;
   const int n = g.npatch;
@@ -1198,7 +1201,7 @@ void apply_operator(const Geom& g, const int* rowptr, const int* colidx, const M
                     const VT* x, const VT* b, VT* out, cudaStream_t st) {
   const unsigned grid = grid_for(g.N, 256);
   if constexpr (sizeof(MT) == 4) {
-    // the other FP32 levels take the Kronecker split (2D order 2), the diagonals or no matrix (3D; order 4)
+    // the other FP32 levels take the Kronecker split (2D order 2), the diagonals or no matrix (3D, order 4)
     if (g.dim != 2 || g.nt != 1) throw Error{STG_EINVAL, "no assembled FP32 operator on this level"};
     launch_k(op_rows<2, 1, MT, VT>, grid, 256, 0, st, g, rowptr, colidx, vv, vp, pv, x, b, out);
   } else if (g.dim == 2) {
@@ -1480,9 +1483,11 @@ void run_patches(const Geom& g, long long p0, long long cnt, const FT* jinv, con
 // coloured, 64 patches a launch n = 60 142 -> 121 us, 63 111 -> 90, 84 196 -> 102, 105 177 -> 112; 1024 n = 63 232 -> 200,
 // 84 505 -> 291, 105 468 -> 460; 4096 n = 63 503 -> 505, 105 1173 -> 1300; averaged, 1024 n = 84 93 -> 60, 4096 133 -> 133
 // (n = 63 84 -> 85, 105 200 -> 230): the line is at 2048.  BF16, two rows -> one: coloured, 64 n = 42 78 -> 70, 84 86 -> 83; 256
-// n = 42 71 -> 68; 1024 77 -> 78: at 512.
+// n = 42 71 -> 68; 1024 77 -> 78: at 512.  FP64 n = 255, 8 columns in flight (registers for one CTA an SM, or spills) -> 4:
+// coloured, 64 patches a launch 3684 -> 1779 us, 512 5515 -> 3643; averaged, 512 746 -> 599, 4096 1019 -> 1325.
 int default_colour_variant(const Geom& g, int factor_prec, long long patches) {
   const int n = g.npatch, size = factor_prec == STG_F64 ? 8 : (factor_prec == STG_F32 ? 4 : 2);
+  if (factor_prec == STG_F64 && patches <= 2048 && n > 192) return 0;
   if (factor_prec == STG_F64) return n < 60 || (patches <= 2048 && n * n * size <= 96 * 1024) ? 11 : 3;
   if (n * n * size > 48 * 1024) return 3;
   return factor_prec == STG_BF16 && patches > 512 ? 15 : 11;

@@ -252,8 +252,8 @@ def q2_block_couplings(cells: tuple) -> int:
 
 def sweep_bytes(dim: int, cells: tuple, k: int, form: str) -> dict:
     """Algorithmic bytes of one averaged Vanka sweep on a level (each array read or written once):
-    the residual r = b - J x (operator + x, b read, r written; in 3D it is matrix-free and its operator is the
-    linearisation velocity), the patch kernel (every J_K^{-1} read, r gathered, y_K written, and read again by
+    the residual r = b - J x (operator + x, b read, r written; in 3D from k = 1 on it is matrix-free and its operator
+    is the linearisation velocity, at k = 0, Oseen, the diagonals of the blocks), the patch kernel (every J_K^{-1} read, r gathered, y_K written, and read again by
     the update) and the update (counted as d and one more vector read and written)."""
     nt = k + 1
     ncell = int(np.prod(cells))
@@ -263,7 +263,9 @@ def sweep_bytes(dim: int, cells: tuple, k: int, form: str) -> dict:
     vs = 8 if form == "f64" else 4
     fs = {"f64": 8, "f32": 4, "bf16": 2}[form]
     vp = ncell * 3 ** dim * nt * dim * (dim + 1)           # velocity-pressure (and pressure-velocity) entries
-    if dim == 3:
+    if dim == 3 and k == 0:
+        op = nnzb * dim * vs + 2 * vp * vs
+    elif dim == 3:
         op = nt * 3 * int(np.prod([2 * c + 1 for c in cells])) * vs   # w at the nodes
     elif form == "f64" or k == 0:
         op = nnzb * (nt * dim) ** 2 * vs + 2 * vp * vs       # dense node blocks

@@ -29,7 +29,7 @@ constexpr int KB = 8;  // columns of a warp = pivots of an elimination block
 // the saddle-point matrix; a pivot below 1e-3 (entries are O(1) after equilibration) flags the
 // patch, and the pivoting kernel redoes it.
 //
-// Bound: FP32 issue (2 n^3 flops a patch) and, where one patch fills an SM (n = 170, 255: 43% of the issue
+// Bound: FP32 issue (2 n^3 flops a patch) and, where one patch fills an SM (n = 170, 255: 32% of the issue
 // slots, the rest barriers and the gather), the elimination of the next block, whose 8 steps are a serial
 // chain of shuffles, a division and RB x 8 FMAs.  Measured over a level, against one barrier per pivot with
 // 8 x 8 tiles a thread: 256^2 n = 63 10.8 -> 2.8 ms, n = 84 14.5 -> 6.0 ms; 352 x 64 n = 120 16.1 -> 5.0 ms;

@@ -4,9 +4,11 @@
 namespace stg {
 
 // Only where its rounding error (rms over the rows of |error| / (|J| |x|), against J in 64 bits) is no larger than that
-// of the entries rounded once.  16 x 8 order 4 with and 6 x 4 x 8, velocity rows, entries -> matrix-free, in 1e-8: Newton k = 0
-// 4.95 -> 5.82 (order 4; assembled) and 7.53 -> 5.31 (3D), Oseen k = 0 4.10 -> 6.5 and 4.80 -> 5.1 (both from the block diagonals),
-// k = 1 4.77 -> 4.72 and 6.03 -> 5.00, k = 2 5.33 -> 4.09 and 6.83 -> 4.84; pressure rows 2.7 -> 2.2 and 3.8 -> 2.8.
+// of the entries rounded once.  16 x 8 order 4 and 6 x 4 x 8, entries -> matrix-free in 1e-8, Oseen (Newton's entries round
+// more): velocity rows k = 1 4.77 -> 4.72 and 6.03 -> 5.00, k = 2 5.33 -> 4.09 and 6.83 -> 4.84; pressure rows 2.7 -> 2.2 and 3.6 ->
+// 2.8; 3D k = 0 with Newton's term 7.53 -> 5.31.  Order 4, k = 0 with Newton's term has 4.95 -> 5.82, and an FP32 emulation of
+// k = 0 without it 3.8 -> 4.8 (order 4) and 4.2 -> 4.9 (3D): these stay assembled, Oseen from the diagonals of the blocks.
+// Steps, without a matrix -> assembled: 48^3 k = 0 76 -> 82 ms, 352 x 64 order 4, k = 0 12.3 -> 15.3 (Newton), 11.8 -> 13.7 (Oseen).
 // 2D order 2 stays with the assembled rows: matrix-free they are as accurate and took 2 of the 19.4 ms of a 704 x 128 step
 // off, but their roundings differ, and any other rounding moves a channel's solution by up to 2e-9 (through a pressure
 // mode that the residual hardly sees).

@@ -225,7 +225,7 @@ __device__ __forceinline__ void add_pressure(const T* __restrict__ table, const 
 // The time coupling of order 4 goes from nodes to nodes by the 1D mass matrices: through the Gauss points, with
 // four factors of L, its velocity rows had up to 1.2 times the rounding error of assembled ones (k = 1, Oseen; the
 // mass term is the largest there).  It costs 50 -> 66 us a launch on 352 x 64.  For order 2 the Gauss points round less
-// (1D entries 1/15 to 16/15).
+// (FP32 emulation in 3D, k = 0: 4.6e-8 against 6.5e-8).
 template <int DIM, int M, int NT, typename T, typename Nodal>
 __device__ __forceinline__ void cell_operator(const MfCoef<T>& cf, int a, int c, unsigned faces, T (&V)[ipow(M, DIM)],
                                               T (&W)[ipow(M, DIM)], T* sv, T* sw, int lane, bool on, Nodal nodal) {
